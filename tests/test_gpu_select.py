@@ -82,3 +82,19 @@ def test_device_arguments_match_host_arguments(R):
                                 True, 20, selected=out)
     assert nc_h == nc_d and t_h == t_d
     np.testing.assert_array_equal(sel_h, sel_d.cpu().numpy())
+
+
+@pytest.mark.parametrize("n,C,thr,lower,upper,adapt", [
+    (4096, 3, 0.9, 1, 1 << 30, False),     # the last size clustered by one CTA
+    (4097, 3, 0.9, 20, 30, True),          # the first by a cluster of 16
+    (31, 128, 9.0, 1, 4, True),            # fewer candidates than a warp, the most CVs
+    (540000, 1, 3.0, 1, 1 << 30, False),   # more than 32 candidates per thread: flag words in memory
+    (540000, 1, 0.5, 2, 3, True),          # the same under a search
+])
+def test_cluster_ownership_edges(R, n, C, thr, lower, upper, adapt):
+    # (equality with the oracle, as above: no tolerance)
+    cv, eps = _frames(n, C, n + C, walkers=1)
+    sel, nc, t = R.select(cv, eps, 0.0, 5.0, thr, lower, upper, adapt, 64)
+    ref = S.select(cv, eps, 0.0, 5.0, thr, lower, upper, adapt, 64)
+    assert (nc, t) == (ref["n_clusters"], ref["threshold"])
+    np.testing.assert_array_equal(sel, ref["selected"])
