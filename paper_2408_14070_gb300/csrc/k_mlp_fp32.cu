@@ -1,244 +1,455 @@
 // k_mlp_fp32.cu -- plain FP32 (SIMT) ensemble MLP: forward pass and
-// reverse-mode input gradient for every member on a tile of 32 walkers.
+// reverse-mode input gradient, or the member values alone, for every member on
+// a tile of R walkers.
 //
-// Grid (ceil(W/32), M), 256 threads.  Warp w owns walkers 8 (w % 4) .. + 7
-// and half (w / 4) of each block of 256 output neurons; a lane takes neurons
-// n = nb + 128 (w / 4) + lane + 32 kk (kk < 4), so a thread keeps an 8 x 4
-// register tile (two warps per SM sub-partition: 8 x 8 tiles on four warps
-// took 261 us per step, this 238 us).  Activations live in shared memory
-// transposed as [neuron][walker] rows of 36 floats (32 walkers + 4 pad:
-// 16-byte aligned rows whose float4 stores by 8 consecutive lanes hit
-// distinct banks).
-// Weight rows (forward: W^T [in][out], backward: W [out][in], 256 output
-// neurons at a time) stream from L2 into a 4-stage ring of 8 rows in shared
-// memory by cp.async, so the eight warps share one copy and three stages are
-// in flight while one is multiplied.  Reading every weight from L2 per warp
-// (four copies, two rows in flight) took 622 us per step of 1024 walkers x
-// 4 x 40-256x4-1; the ring takes 263 us.
-// tanh(z_l) of every layer is kept in a global scratch [M][tile][L][32][H]
+// Grid (ceil(W / R), M), 256 threads: 8 / WCN warp rows x WCN warp columns of
+// 128 output neurons, WCN = 1, 2 or 4 by width, so a layer is one pass over
+// its inputs.  In a warp, half (lane / 16) takes one group of RPT walkers and
+// lane % 16 the columns 4 lc .. + 3 and 64 + 4 lc .. + 3, so a thread keeps an
+// RPT x 8 register tile, accumulated by fma.rn.f32x2 (two neighbouring columns
+// an instruction; each half rounds as fmaf does).  Activations live in shared
+// memory transposed as [neuron][walker] rows of LD floats, one group of RPT
+// walkers in GS slots (RPT rounded up to a power of two), so a thread's walkers
+// are one or two 16-byte loads; a layer's outputs go back over its inputs once
+// every warp has read them.
+// Weight rows (forward: W^T [in][out], backward: W [out][in]) stream from L2
+// into a ring of NSW stages of KC rows in shared memory by cp.async, shared by
+// the eight warps, the first stages of a layer during the epilogue of the one
+// before it.
+// tanh(z_l) of every layer is kept in a global scratch [M][tile][L][H][slots]
 // (L2-resident at the sizes used) for the backward pass:
 //   g_L = w_out,  delta_l = g_l * (1 - tanh^2 z_l),
 //   g_{l-1} = W_l^T delta_l (+ g_l for a residual layer),
 //   dA/ds_j = -sin s_j g_0[2j] + cos s_j g_0[2j+1].
+//
+// Bound by the FP32 pipe at RPT >= 4 (one CTA an SM, two warps a scheduler; a K
+// row is 16 RPT cycles of FMAs and 40 to 48 of shared loads), by the shared loads
+// at RPT = 2.  The walker count of a tile follows the call (choose_rpt).
+// 1024 walkers x 4 members 40-256x4-1 (128 tiles of 32): 238 us with a 256-thread
+// CTA of 8 x 4 register tiles, scalar FMAs and 8-row stages, 115 us now (29.5 of
+// 69.8 TFLOP/s); a force evaluation of them 353 -> 237 us.
 #include "rid_internal.cuh"
 
 namespace {
 
-constexpr int TW = 32;    // walkers per CTA
-constexpr int ROW = 36;   // shared row stride in floats
-constexpr int NT = 256;   // threads per CTA: warp w takes walkers 8 (w % 4) .. and neuron half w / 4
-constexpr int NK = 4;     // neuron columns per thread (of 32 lanes apart)
-
-constexpr int KC = 8;     // weight rows per ring stage
-constexpr int NSW = 4;    // ring stages
-constexpr int WCOLS = 256;
+constexpr int NT = 256;   // threads per CTA
+constexpr int F32_SMEM_MAX = 227 * 1024;
 
 __device__ __forceinline__ void cpa4(float* dst, const float* src, int bytes) {
     const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(d), "l"(src), "r"(bytes) : "memory");
 }
-__device__ __forceinline__ void cpa16(float* dst, const float* src, int bytes) {
+__device__ __forceinline__ void cpa16(float* dst, const float* src) {
     const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "r"(bytes) : "memory");
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cpa_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cpa_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
-// acc[i][kk] += sum_k in[k][8 (warp % 4) + i] * Wg[k * ldw + nb + 128 (warp / 4) + lane + 32 kk]
-// The CTA's weight rows stream through a ring of NSW stages of KC rows x 256
-// columns in shared memory (ws), so the eight warps share one copy; every
-// accumulator still sums its K terms in increasing order.
-__device__ __forceinline__ void tile_gemm(const float* __restrict__ in, int K, const float* __restrict__ Wg, int ldw,
-                                          int N, int nb, int warp, int lane, float (&acc)[8][NK], float* ws) {
-    const int wg = warp & 3, nh = (warp >> 2) * 32 * NK;   // walker group, neuron offset within the block
-    const int nst = (K + KC - 1) / KC;
-    const int ncol = N - nb < WCOLS ? N - nb : WCOLS;
-    const bool vec = (ldw & 3) == 0 && (nb & 3) == 0 && (reinterpret_cast<uintptr_t>(Wg) & 15) == 0;
-    auto issue = [&](int t) {
-        if (t < nst) {
-            float* dst = ws + (t % NSW) * KC * WCOLS;
-            const int k0 = t * KC;
-            if (vec) {
-                for (int q = threadIdx.x; q < KC * WCOLS / 4; q += NT) {
-                    const int r = q / (WCOLS / 4), c4 = 4 * (q % (WCOLS / 4)), k = k0 + r;
-                    int valid = k < K ? ncol - c4 : 0;
-                    valid = valid < 0 ? 0 : (valid > 4 ? 4 : valid);
-                    cpa16(dst + r * WCOLS + c4, valid ? Wg + (size_t)k * ldw + nb + c4 : Wg, 4 * valid);
-                }
-            } else {
-                for (int q = threadIdx.x; q < KC * WCOLS; q += NT) {
-                    const int r = q / WCOLS, c = q % WCOLS, k = k0 + r;
-                    const bool ok = k < K && c < ncol;
-                    cpa4(dst + r * WCOLS + c, ok ? Wg + (size_t)k * ldw + nb + c : Wg, ok ? 4 : 0);
-                }
+// Two FP32 values in one 64-bit register pair, and their fused multiply-add.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ void fma2(f32x2& acc, f32x2 a, f32x2 b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+
+// Tile shape: RPT walkers a thread, WCN warp columns.
+template <int RPT, int WCN>
+struct Shape {
+    static constexpr int GS = RPT > 4 ? 8 : RPT > 2 ? 4 : RPT;   // slots of a walker group
+    static constexpr int GROUPS = 2 * (8 / WCN);                 // walker groups of a CTA
+    static constexpr int R = GROUPS * RPT;                       // walkers of a CTA
+    static constexpr int SLOTS = GROUPS * GS;
+    static constexpr int LD = SLOTS + 4;                         // floats of a shared row
+    static constexpr int COLS = 128 * WCN;                       // output neurons
+    // weight rows per ring stage: 32 KB a stage (16 rows of 256 columns cost 84 us where 32 cost
+    // 78, for twice the block barriers); short tiles, whose rows are consumed faster than one
+    // stage ahead arrives, keep more stages
+    static constexpr int KC = WCN == 4 ? 16 : 32;
+    static constexpr int NSW = RPT <= 2 ? 4 : 2;
+};
+__host__ __device__ constexpr int shape_gs(int rpt) { return rpt > 4 ? 8 : rpt > 2 ? 4 : rpt; }
+
+// Shared memory of a tile, bytes: activations (and, for a residual gradient, g_l
+// beside them), the inputs, the weight ring.
+size_t tile_smem(int rpt, int wcn, int D, int H, int resnet, bool bwd) {
+    const int slots = 2 * (8 / wcn) * shape_gs(rpt), ld = slots + 4;
+    const int kc = wcn == 4 ? 16 : 32, nsw = rpt <= 2 ? 4 : 2;
+    return sizeof(float) * ((size_t)(bwd && resnet ? 2 : 1) * H * ld + (size_t)D * ld + (size_t)nsw * kc * 128 * wcn);
+}
+
+// Where a thread's outputs lie: walker group, column base of its warp.
+struct Lane {
+    int rg, lc, wc;
+};
+template <int WCN>
+__device__ __forceinline__ Lane lane_of() {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    return Lane{(warp / WCN) * 2 + (lane >> 4), lane & 15, warp % WCN};
+}
+// Column j (0..7) of a thread within a pass.
+__device__ __forceinline__ int col_of(const Lane& t, int j) {
+    return 128 * t.wc + (j < 4 ? 4 * t.lc + j : 64 + 4 * t.lc + j - 4);
+}
+
+// The RPT values of a walker group at p (GS slots, aligned to them).
+template <int RPT>
+__device__ __forceinline__ void load_group(const float* p, float (&v)[RPT]) {
+    constexpr int GS = shape_gs(RPT);
+    float t[GS];
+    if constexpr (GS >= 4) {
+#pragma unroll
+        for (int q = 0; q < GS / 4; ++q) {
+            const float4 a = *reinterpret_cast<const float4*>(p + 4 * q);
+            t[4 * q] = a.x, t[4 * q + 1] = a.y, t[4 * q + 2] = a.z, t[4 * q + 3] = a.w;
+        }
+    } else if constexpr (GS == 2) {
+        const float2 a = *reinterpret_cast<const float2*>(p);
+        t[0] = a.x, t[1] = a.y;
+    } else {
+        t[0] = *p;
+    }
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) v[i] = t[i];
+}
+template <int RPT>
+__device__ __forceinline__ void store_group(float* p, const float (&v)[RPT]) {
+    constexpr int GS = shape_gs(RPT);
+    float t[GS];
+#pragma unroll
+    for (int i = 0; i < GS; ++i) t[i] = i < RPT ? v[i < RPT ? i : 0] : 0.0f;
+    if constexpr (GS >= 4) {
+#pragma unroll
+        for (int q = 0; q < GS / 4; ++q)
+            *reinterpret_cast<float4*>(p + 4 * q) = make_float4(t[4 * q], t[4 * q + 1], t[4 * q + 2], t[4 * q + 3]);
+    } else if constexpr (GS == 2) {
+        *reinterpret_cast<float2*>(p) = make_float2(t[0], t[1]);
+    } else {
+        *p = t[0];
+    }
+}
+
+// The weight rows of one pass: K rows of ldw floats from W on, whose first
+// `ncol` columns are loaded (vec: a multiple of 4 with 16-byte aligned rows) and
+// whose first `nuse` are wanted.
+struct Stream {
+    const float* W;
+    int K, ldw, ncol, nuse;
+    bool vec;
+};
+template <typename S>
+__device__ __forceinline__ void ring_issue(const Stream& q, int st, float* ws) {
+    constexpr int KC = S::KC, COLS = S::COLS, NSW = S::NSW;
+    const int kn = q.K - st * KC < KC ? q.K - st * KC : KC;
+    if (kn > 0) {
+        float* dst = ws + (st % NSW) * KC * COLS;
+        const float* src = q.W + (size_t)st * KC * q.ldw;
+        if (q.vec) {
+#pragma unroll
+            for (int e = threadIdx.x; e < KC * COLS / 4; e += NT) {
+                const int r = e / (COLS / 4), c = 4 * (e % (COLS / 4));
+                if (r < kn && c < q.ncol) cpa16(dst + r * COLS + c, src + (size_t)r * q.ldw + c);
+            }
+        } else {
+            for (int e = threadIdx.x; e < KC * COLS; e += NT) {
+                const int r = e / COLS, c = e % COLS;
+                if (r < kn && c < q.ncol) cpa4(dst + r * COLS + c, src + (size_t)r * q.ldw + c, 4);
             }
         }
-        cpa_commit();
-    };
+    }
+    cpa_commit();
+}
+// The first stages of a pass; the ring must be free.
+template <typename S>
+__device__ __forceinline__ void ring_prime(const Stream& q, float* ws) {
 #pragma unroll
-    for (int t = 0; t < NSW - 1; ++t) issue(t);
-    for (int t = 0; t < nst; ++t) {
+    for (int st = 0; st < S::NSW - 1; ++st) ring_issue<S>(q, st, ws);
+}
+
+// acc[i][j] += sum_k in[k][walker i] * W[k][column j] for a primed pass, every
+// accumulator over k in increasing order.  SPLIT sums the K tiles of 32 with
+// even and odd index in acc and acc1.  Ends with every warp past its last read
+// of `in` and of the ring.
+template <int RPT, int WCN, bool SPLIT>
+__device__ __forceinline__ void tile_gemm(const float* in, const Stream& q, const Lane& t, f32x2 (&acc)[RPT][4],
+                                          f32x2 (&acc1)[SPLIT ? RPT : 1][4], float* ws) {
+    using S = Shape<RPT, WCN>;
+    constexpr int KC = S::KC, COLS = S::COLS, NSW = S::NSW;
+    const int nst = (q.K + KC - 1) / KC;
+    const bool use = 128 * t.wc < q.nuse;    // warp-uniform: some column of this warp is wanted
+    auto stage = [&](int st, f32x2(&a)[RPT][4]) {
+        const float* wsr = ws + (st % NSW) * KC * COLS + 128 * t.wc + 4 * t.lc;
+        const float* ar = in + (size_t)st * KC * S::LD + t.rg * S::GS;
+        const int kn = q.K - st * KC < KC ? q.K - st * KC : KC;
+        auto row = [&](int r) {
+            float av[RPT];
+            load_group<RPT>(ar + r * S::LD, av);
+            const ulonglong2 w0 = *reinterpret_cast<const ulonglong2*>(wsr + r * COLS);
+            const ulonglong2 w1 = *reinterpret_cast<const ulonglong2*>(wsr + r * COLS + 64);
+#pragma unroll
+            for (int i = 0; i < RPT; ++i) {
+                const f32x2 d = pack2(av[i], av[i]);
+                fma2(a[i][0], d, w0.x);
+                fma2(a[i][1], d, w0.y);
+                fma2(a[i][2], d, w1.x);
+                fma2(a[i][3], d, w1.y);
+            }
+        };
+        if (kn == KC) {
+#pragma unroll
+            for (int r = 0; r < KC; ++r) row(r);
+        } else {
+            for (int r = 0; r < kn; ++r) row(r);
+        }
+    };
+    for (int st = 0; st < nst; ++st) {
         cpa_wait<NSW - 2>();
         __syncthreads();
-        issue(t + NSW - 1);
-        const float* wsr = ws + (t % NSW) * KC * WCOLS + nh + lane;
-        const int kn = K - t * KC < KC ? K - t * KC : KC;
-#pragma unroll 4
-        for (int r = 0; r < kn; ++r) {
-            const int k = t * KC + r;
-            const float4 a0 = *reinterpret_cast<const float4*>(in + k * ROW + 8 * wg);
-            const float4 a1 = *reinterpret_cast<const float4*>(in + k * ROW + 8 * wg + 4);
-            const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-            float wv[NK];
-#pragma unroll
-            for (int kk = 0; kk < NK; ++kk) wv[kk] = wsr[r * WCOLS + 32 * kk];
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-#pragma unroll
-                for (int kk = 0; kk < NK; ++kk) acc[i][kk] = fmaf(a[i], wv[kk], acc[i][kk]);
+        ring_issue<S>(q, st + NSW - 1, ws);
+        if (use) {
+            if constexpr (SPLIT) {
+                if ((st * KC / 32) & 1) stage(st, acc1);
+                else stage(st, acc);
+            } else {
+                stage(st, acc);
+            }
         }
     }
     cpa_wait<0>();
-    __syncthreads();   // the ring is refilled by the next call
+    __syncthreads();
 }
 
-__global__ void __launch_bounds__(NT) k_mlp_fp32(EnsDev E, StateDev st, int W, int C) {
+// BWD: the input gradient as well; else the member values alone.
+template <int RPT, int WCN, bool BWD, bool SPLIT>
+__global__ void __launch_bounds__(NT, RPT >= 4 ? 1 : 2) k_mlp_fp32(MlpF32 E) {
+    using S = Shape<RPT, WCN>;
+    constexpr int GS = S::GS, LD = S::LD, R = S::R;
     extern __shared__ __align__(16) float sm[];
-    const int D = E.D, L = E.L, H = E.H, M = E.M;
-    const int Kmax = H > D ? H : D;
-    float* bufA = sm;
-    float* bufB = bufA + Kmax * ROW;
-    float* ubuf = bufB + Kmax * ROW;
-    float* ws = ubuf + D * ROW;   // weight ring [NSW][KC][256]
+    const int D = E.D, L = E.L, H = E.H, W = E.W;
+    float* X = sm;                                      // current activations, then delta_l  [H][LD]
+    float* Y = X + (size_t)(BWD && E.resnet ? H : 0) * LD;   // g_l (residual gradient)          [H][LD]
+    float* ubuf = Y + (size_t)H * LD;
+    float* ws = ubuf + (size_t)D * LD;                  // weight ring [NSW][KC][COLS]
     const int m = blockIdx.y, tile = blockIdx.x, ntiles = gridDim.x;
-    const int w0 = tile * TW;
+    const int w0 = tile * R;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int wgp = warp & 3, nh = (warp >> 2) * 32 * NK;   // walker group, neuron offset in a block
-    const float* Wm = E.W + (size_t)m * E.wstride;
-    const float* WTm = E.WT + (size_t)m * E.wstride;
-    float* hs = st.hs + ((size_t)m * ntiles + tile) * (size_t)L * TW * H;
+    const Lane t = lane_of<WCN>();
+    float* hs = BWD ? E.hs + ((size_t)m * ntiles + tile) * (size_t)L * H * S::SLOTS : nullptr;
+    const int own = t.rg * GS;                          // this thread's slots of a row
 
-    for (int idx = threadIdx.x; idx < D * TW; idx += NT) {
-        const int wl = idx / D, k = idx - wl * D;
-        ubuf[k * ROW + wl] = (w0 + wl < W) ? st.u[(size_t)(w0 + wl) * D + k] : 0.0f;
+    // the passes in order: forward layers, then (BWD) gradient layers L - 1 .. 0
+    const int npass = BWD ? 2 * L : L;
+    auto stream = [&](int p) {
+        Stream q{};
+        if (p >= npass) return q;
+        if (p < L) {
+            q.W = E.WT + (long long)m * E.wt_st + E.toff[p];
+            q.K = p == 0 ? D : H;
+            q.ldw = q.ncol = E.ldt;
+            q.nuse = H;
+            q.vec = true;
+        } else {
+            const int l = 2 * L - 1 - p;
+            q.W = E.Wb + (long long)m * E.wb_st + E.woff[l];   // [H][fin] row-major = [K][Nout]
+            q.K = H;
+            q.ldw = q.ncol = q.nuse = l == 0 ? D : H;
+            q.vec = (q.ldw & 3) == 0 && (reinterpret_cast<uintptr_t>(q.W) & 15) == 0;
+        }
+        return q;
+    };
+    int pass = 0;
+    Stream cur = stream(0);
+    ring_prime<S>(cur, ws);
+    auto next_pass = [&]() {
+        cur = stream(++pass);
+        ring_prime<S>(cur, ws);
+    };
+
+    for (int idx = threadIdx.x; idx < D * R; idx += NT) {
+        const int r = idx / D, k = idx - r * D;
+        ubuf[k * LD + (r / RPT) * GS + r % RPT] = (w0 + r < W) ? E.u[(size_t)(w0 + r) * D + k] : 0.0f;
     }
     __syncthreads();
 
+    f32x2 acc1[SPLIT ? RPT : 1][4];
+    // value (i, j) of an accumulator set
+    auto value = [](const f32x2(&a)[RPT][4], int i, int j) {
+        float lo, hi;
+        unpack2(a[i][j >> 1], lo, hi);
+        return (j & 1) ? hi : lo;
+    };
     // ---------------- forward
-    const float* in = ubuf;
-    float* out = bufA;
     for (int l = 0; l < L; ++l) {
-        const int K = l == 0 ? D : H;
-        const float* Wt = WTm + E.loff[l];
-        const float* bias = E.b + ((size_t)m * L + l) * H;
-        for (int nb = 0; nb < H; nb += 256) {
-            float acc[8][NK];
+        const float* bias = E.b + (long long)m * E.b_st + E.boff[l];
+        f32x2 acc[RPT][4];
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
+        for (int i = 0; i < RPT; ++i)
 #pragma unroll
-                for (int kk = 0; kk < NK; ++kk) acc[i][kk] = 0.0f;
-            tile_gemm(in, K, Wt, H, H, nb, warp, lane, acc, ws);
+            for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+        if constexpr (SPLIT)
 #pragma unroll
-            for (int kk = 0; kk < NK; ++kk) {
-                const int n = nb + nh + lane + 32 * kk;
-                if (n < H) {
-                    const float bn = bias[n];
-                    float h[8];
+            for (int i = 0; i < RPT; ++i)
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const float t = tanhf(acc[i][kk] + bn);
-                        hs[((size_t)l * TW + 8 * wgp + i) * H + n] = t;
-                        h[i] = (E.resnet && l > 0) ? t + in[n * ROW + 8 * wgp + i] : t;
+                for (int j = 0; j < 4; ++j) acc1[i][j] = 0ull;
+        tile_gemm<RPT, WCN, SPLIT>(l == 0 ? ubuf : X, cur, t, acc, acc1, ws);
+        next_pass();
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int n = col_of(t, j);
+            if (n < H) {
+                const float bn = bias[n];
+                float tv[RPT], h[RPT];
+#pragma unroll
+                for (int i = 0; i < RPT; ++i) {
+                    float z = value(acc, i, j);
+                    if constexpr (SPLIT) z += value(acc1, i, j);
+                    tv[i] = tanhf(z + bn);
+                }
+                if (BWD) store_group<RPT>(hs + ((size_t)l * H + n) * S::SLOTS + own, tv);
+                if (E.resnet && l > 0) {
+                    load_group<RPT>(X + (size_t)n * LD + own, h);
+#pragma unroll
+                    for (int i = 0; i < RPT; ++i) h[i] = tv[i] + h[i];
+                    store_group<RPT>(X + (size_t)n * LD + own, h);
+                } else {
+                    store_group<RPT>(X + (size_t)n * LD + own, tv);
+                }
+            }
+        }
+        __syncthreads();
+    }
+    // value A = w_out . h_L + b_out: lane-strided partial sums, then the butterfly
+    const float* wo = E.wout + (long long)m * E.wo_st;
+    for (int r = warp; r < R; r += NT / 32) {
+        if (w0 + r >= W) break;
+        const float* hr = X + (r / RPT) * GS + r % RPT;
+        float part = 0.0f;
+        for (int n = lane; n < H; n += 32) part = fmaf(wo[n], hr[(size_t)n * LD], part);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+        if (lane == 0) E.Aval[(size_t)m * W + w0 + r] = part + E.bout[(long long)m * E.bo_st];
+    }
+    if constexpr (BWD) {
+        // ---------------- backward: X holds delta_l, Y g_l of this thread's own columns
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int n = col_of(t, j);
+            if (n < H) {
+                const float wn = wo[n];
+                float tv[RPT], g[RPT];
+                load_group<RPT>(hs + ((size_t)(L - 1) * H + n) * S::SLOTS + own, tv);
+#pragma unroll
+                for (int i = 0; i < RPT; ++i) {
+                    g[i] = wn;
+                    tv[i] = wn * (1.0f - tv[i] * tv[i]);
+                }
+                store_group<RPT>(X + (size_t)n * LD + own, tv);
+                if (E.resnet) store_group<RPT>(Y + (size_t)n * LD + own, g);
+            }
+        }
+        __syncthreads();
+        for (int l = L - 1; l >= 0; --l) {
+            const bool res = E.resnet && l > 0;
+            f32x2 acc[RPT][4];
+            float g[RPT][8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int n = col_of(t, j);
+                float v[RPT];
+                if (res && n < H) load_group<RPT>(Y + (size_t)n * LD + own, v);
+#pragma unroll
+                for (int i = 0; i < RPT; ++i) g[i][j] = res && n < H ? v[i] : 0.0f;
+            }
+#pragma unroll
+            for (int i = 0; i < RPT; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = pack2(g[i][2 * j], g[i][2 * j + 1]);
+            tile_gemm<RPT, WCN, false>(X, cur, t, acc, acc1, ws);
+            next_pass();
+#pragma unroll
+            for (int i = 0; i < RPT; ++i)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) g[i][j] = value(acc, i, j);
+            if (l > 0) {
+                // g_{l-1}, and its delta over delta_l
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int n = col_of(t, j);
+                    if (n >= H) continue;
+                    float v[RPT], tv[RPT];
+                    load_group<RPT>(hs + ((size_t)(l - 1) * H + n) * S::SLOTS + own, tv);
+#pragma unroll
+                    for (int i = 0; i < RPT; ++i) v[i] = g[i][j];
+                    if (E.resnet) store_group<RPT>(Y + (size_t)n * LD + own, v);
+#pragma unroll
+                    for (int i = 0; i < RPT; ++i) v[i] = v[i] * (1.0f - tv[i] * tv[i]);
+                    store_group<RPT>(X + (size_t)n * LD + own, v);
+                }
+                __syncthreads();
+            } else {
+                // dA/ds_j = -sin s_j g0[2j] + cos s_j g0[2j+1] (torsion), g0[2j] (distance: input (s, 0))
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int n = col_of(t, 2 * q), j = n >> 1;
+                    if (n >= D) continue;
+                    const bool dist = E.cvdist && __ldg(E.cvdist + j);
+                    float cs[RPT], sn[RPT];
+                    load_group<RPT>(ubuf + (size_t)n * LD + own, cs);
+                    load_group<RPT>(ubuf + (size_t)(n + 1) * LD + own, sn);
+#pragma unroll
+                    for (int i = 0; i < RPT; ++i) {
+                        const int wg = w0 + t.rg * RPT + i;
+                        const float G0 = g[i][2 * q], G1 = g[i][2 * q + 1];
+                        const float gr = dist ? G0 : -sn[i] * G0 + cs[i] * G1;
+                        if (wg < W) E.gradA[((size_t)m * W + wg) * E.C + j] = gr;
                     }
-                    *reinterpret_cast<float4*>(out + n * ROW + 8 * wgp) = make_float4(h[0], h[1], h[2], h[3]);
-                    *reinterpret_cast<float4*>(out + n * ROW + 8 * wgp + 4) = make_float4(h[4], h[5], h[6], h[7]);
                 }
             }
         }
-        __syncthreads();
-        in = out;
-        out = (out == bufA) ? bufB : bufA;
     }
-    // value A = w_out . h_L + b_out (warps 0-3, one per walker group)
-    if (warp < 4) {
-        const float* wo = E.wout + (size_t)m * H;
-        float part[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        for (int n = lane; n < H; n += 32) {
-            const float wn = wo[n];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) part[i] = fmaf(wn, in[n * ROW + 8 * warp + i], part[i]);
-        }
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) part[i] += __shfl_xor_sync(0xffffffffu, part[i], o);
-        }
-        if (lane == 0) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int wg = w0 + 8 * warp + i;
-                if (wg < W) st.Aval[(size_t)m * W + wg] = part[i] + E.bout[m];
-            }
-        }
-    }
-    // ---------------- backward: G holds g_l, Dl holds delta_l
-    float* G = (in == bufA) ? bufB : bufA;   // free buffer
-    float* Dl = (float*)in;                  // h_L no longer needed
-    {
-        const float* wo = E.wout + (size_t)m * H;
-        for (int idx = threadIdx.x; idx < H * TW; idx += NT) {
-            const int n = idx / TW, wl = idx - n * TW;
-            G[n * ROW + wl] = wo[n];
+}
+
+// Walkers per thread: the tile whose waves of CTAs over the SMs cost least,
+// counting a K row at the larger of its FMA cycles (16 RPT) and its shared loads
+// (40), plus 8 for what does not overlap; of those that fit in shared memory.
+// Two walkers always fit.
+int choose_rpt(int wcn, int W, int M, int D, int H, int resnet, bool bwd) {
+    static int nsm[64] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) dev = 0;
+    int& n = nsm[dev & 63];
+    if (n == 0 && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) n = 152;
+    int best = 2;
+    long long cost = -1;
+    for (int rpt : {2, 4, 7, 8}) {
+        if (tile_smem(rpt, wcn, D, H, resnet, bwd) > (size_t)F32_SMEM_MAX) continue;
+        const int R = 2 * (8 / wcn) * rpt;
+        const long long ctas = (long long)((W + R - 1) / R) * M;
+        const long long c = (ctas + n - 1) / n * ((16 * rpt > 40 ? 16 * rpt : 40) + 8);
+        if (cost < 0 || c <= cost) {
+            cost = c;
+            best = rpt;
         }
     }
-    __syncthreads();
-    for (int l = L - 1; l >= 0; --l) {
-        const int K = H, Nout = l == 0 ? D : H;
-        // delta_l = g_l * (1 - t_l^2)
-        for (int idx = threadIdx.x; idx < H * TW; idx += NT) {
-            const int wl = idx / H, n = idx - wl * H;
-            const float t = hs[((size_t)l * TW + wl) * H + n];
-            Dl[n * ROW + wl] = G[n * ROW + wl] * (1.0f - t * t);
-        }
-        __syncthreads();
-        const float* Wl = Wm + E.loff[l];   // [H][fin] row-major = [K][Nout]
-        const bool res = E.resnet && l > 0;
-        float accs[8][NK];
-        for (int nb = 0; nb < Nout; nb += 256) {
-#pragma unroll
-            for (int kk = 0; kk < NK; ++kk) {
-                const int n = nb + nh + lane + 32 * kk;
-#pragma unroll
-                for (int i = 0; i < 8; ++i) accs[i][kk] = (res && n < Nout) ? G[n * ROW + 8 * wgp + i] : 0.0f;
-            }
-            tile_gemm(Dl, K, Wl, Nout, Nout, nb, warp, lane, accs, ws);
-            __syncthreads();   // every thread has read G for its initial values
-#pragma unroll
-            for (int kk = 0; kk < NK; ++kk) {
-                const int n = nb + nh + lane + 32 * kk;
-                if (n < Nout) {
-                    *reinterpret_cast<float4*>(G + n * ROW + 8 * wgp) =
-                        make_float4(accs[0][kk], accs[1][kk], accs[2][kk], accs[3][kk]);
-                    *reinterpret_cast<float4*>(G + n * ROW + 8 * wgp + 4) =
-                        make_float4(accs[4][kk], accs[5][kk], accs[6][kk], accs[7][kk]);
-                }
-            }
-        }
-        __syncthreads();
-    }
-    // dA/ds_j = -sin s_j g0[2j] + cos s_j g0[2j+1] (torsion), g0[2j] (distance: input (s, 0))
-    for (int idx = threadIdx.x; idx < C * TW; idx += NT) {
-        const int wl = idx / C, j = idx - wl * C;
-        const int wg = w0 + wl;
-        if (wg < W) {
-            const float cs = ubuf[(2 * j) * ROW + wl], sn = ubuf[(2 * j + 1) * ROW + wl];
-            const bool dist = E.cvdist && __ldg(E.cvdist + j);
-            const float g = dist ? G[(2 * j) * ROW + wl] : -sn * G[(2 * j) * ROW + wl] + cs * G[(2 * j + 1) * ROW + wl];
-            st.gradA[((size_t)m * W + wg) * C + j] = g;
-        }
-    }
-    (void)M;
+    return best;
+}
+
+template <int RPT, int WCN, bool BWD, bool SPLIT>
+void launch_f32(const MlpF32& E, int M, cudaStream_t s) {
+    static unsigned long long attr = 0;
+    auto k = k_mlp_fp32<RPT, WCN, BWD, SPLIT>;
+    if (rid_first_on_device(attr)) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, F32_SMEM_MAX);
+    constexpr int R = Shape<RPT, WCN>::R;
+    k<<<dim3((E.W + R - 1) / R, M), NT, tile_smem(RPT, WCN, E.D, E.H, E.resnet, BWD), s>>>(E);
 }
 
 // Small ensembles (every layer of a member fits in shared memory at once, as
@@ -253,7 +464,7 @@ __global__ void __launch_bounds__(NT) k_mlp_fp32(EnsDev E, StateDev st, int W, i
 // the member value is the same lane-strided partial sums and butterfly.
 constexpr int SM_MAX_FLOATS = 50 * 1024;   // 200 KB of shared memory
 constexpr int SM_MAX_WIDTH = 128;          // at least two walker groups per neuron
-constexpr int SR_MAX = TW / (NT / SM_MAX_WIDTH);   // walkers per thread at the widest layer: 16
+constexpr int SR_MAX = 32 / (NT / SM_MAX_WIDTH);   // walkers per thread at the widest layer: 16
 
 struct SmallLayout {
     int woff[RID_MAX_LAYERS + 1];
@@ -415,19 +626,41 @@ __global__ void __launch_bounds__(NT) k_mlp_fp32_small(EnsDev E, StateDev st, in
 
 }  // namespace
 
-size_t rid_mlp_fp32_scratch_floats(int W, int M, int L, int H) {
-    const size_t ntiles = (size_t)(W + TW - 1) / TW;
-    return (size_t)M * ntiles * L * TW * H;
-}
-
-void rid_launch_mlp_fp32(const EnsDev& E, StateDev st, int W, int C, cudaStream_t s) {
-    // walkers per CTA: the largest power of two up to 32 that still gives one
-    // wave of CTAs (152 SMs), at least one walker
+// The small kernel's walkers per CTA for this call, 0 when it does not apply:
+// the largest power of two up to 32 that still gives one wave of CTAs.
+static int small_tile(const EnsDev& E, int W) {
+    if (E.H > SM_MAX_WIDTH || E.D > NT || small_layout(E.D, E.L, E.H, E.resnet, 32).total > SM_MAX_FLOATS) return 0;
     int tw = 32;
     while (tw > 1 && (long long)((W + tw - 1) / tw) * E.M < 152) tw >>= 1;
-    const SmallLayout Y = small_layout(E.D, E.L, E.H, E.resnet, tw);
-    if (Y.total <= SM_MAX_FLOATS && small_layout(E.D, E.L, E.H, E.resnet, 32).total <= SM_MAX_FLOATS &&
-        E.H <= SM_MAX_WIDTH && E.D <= NT) {
+    return tw;
+}
+
+// Rounded up over every tile shape (7 walkers take 8 slots), so that it grows
+// with W: a system keeps the scratch of its largest walker count.
+size_t rid_mlp_fp32_scratch_floats(const EnsDev& E, int W) {
+    return (size_t)E.M * E.L * E.H * ((size_t)(W + 27) / 28 * 32 + 64);
+}
+
+// The kernel for a width, walkers per thread chosen.
+template <int WCN, bool BWD, bool SPLIT>
+static void launch_shape(const MlpF32& E, int M, cudaStream_t s) {
+    switch (choose_rpt(WCN, E.W, M, E.D, E.H, E.resnet, BWD)) {
+        case 2: return launch_f32<2, WCN, BWD, SPLIT>(E, M, s);
+        case 4: return launch_f32<4, WCN, BWD, SPLIT>(E, M, s);
+        case 7: return launch_f32<7, WCN, BWD, SPLIT>(E, M, s);
+        default: return launch_f32<8, WCN, BWD, SPLIT>(E, M, s);
+    }
+}
+template <bool SPLIT>
+static void launch_values(const MlpF32& E, int M, cudaStream_t s) {
+    if (E.H <= 128) launch_shape<1, false, SPLIT>(E, M, s);
+    else if (E.H <= 256) launch_shape<2, false, SPLIT>(E, M, s);
+    else launch_shape<4, false, SPLIT>(E, M, s);
+}
+
+void rid_launch_mlp_fp32(const EnsDev& E, StateDev st, int W, int C, cudaStream_t s, bool values_only) {
+    if (const int tw = small_tile(E, W)) {
+        const SmallLayout Y = small_layout(E.D, E.L, E.H, E.resnet, tw);
         const int wpt = (tw + NT / E.H - 1) / (NT / E.H);
         int sr = 1;
         while (sr < wpt) sr <<= 1;
@@ -441,13 +674,38 @@ void rid_launch_mlp_fp32(const EnsDev& E, StateDev st, int W, int C, cudaStream_
         kern<<<dim3((W + tw - 1) / tw, E.M), NT, (size_t)Y.total * sizeof(float), s>>>(E, st, W, C, tw);
         return;
     }
-    const int Kmax = E.H > E.D ? E.H : E.D;
-    const size_t sm = sizeof(float) * ((size_t)2 * Kmax * ROW + (size_t)E.D * ROW + (size_t)NSW * KC * WCOLS);
-    static unsigned long long attr_set = 0;
-    if (rid_first_on_device(attr_set)) {
-        // activations 2 x 512 x 36 + inputs 256 x 36 + ring 4 x 8 x 256 floats = 212 KB at the limits
-        cudaFuncSetAttribute(k_mlp_fp32, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    MlpF32 A{};
+    A.WT = E.WT;
+    A.Wb = E.W;
+    A.wt_st = A.wb_st = E.wstride;
+    A.ldt = E.H;
+    A.b = E.b;
+    A.b_st = (long long)E.L * E.H;
+    for (int l = 0; l < E.L; ++l) {
+        A.toff[l] = A.woff[l] = E.loff[l];
+        A.boff[l] = (long long)l * E.H;
     }
-    dim3 grid((W + TW - 1) / TW, E.M);
-    k_mlp_fp32<<<grid, NT, sm, s>>>(E, st, W, C);
+    A.wout = E.wout;
+    A.wo_st = E.H;
+    A.bout = E.bout;
+    A.bo_st = 1;
+    A.u = st.u;
+    A.D = E.D;
+    A.L = E.L;
+    A.H = E.H;
+    A.resnet = E.resnet;
+    A.W = W;
+    A.C = C;
+    A.hs = st.hs;
+    A.Aval = st.Aval;
+    A.gradA = st.gradA;
+    A.cvdist = E.cvdist;
+    if (values_only) launch_values<false>(A, E.M, s);
+    else if (E.H <= 256) launch_shape<2, true, false>(A, E.M, s);
+    else launch_shape<4, true, false>(A, E.M, s);
+}
+
+void rid_launch_mlp_values(const MlpF32& E, int M, bool split, cudaStream_t s) {
+    if (split) launch_values<true>(E, M, s);
+    else launch_values<false>(E, M, s);
 }

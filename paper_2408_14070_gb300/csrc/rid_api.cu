@@ -233,7 +233,7 @@ static int ensure_state(rid_system* sys, int W) {
         TRY(sys->Aval.ensure((size_t)E.M * W * sizeof(float)));
         TRY(sys->Aval.ensure((size_t)E.M * W * sizeof(float)));
         if (sys->precision == RID_PREC_FP32) {
-            TRY(sys->hs.ensure(rid_mlp_fp32_scratch_floats(W, E.M, E.L, E.H) * sizeof(float)));
+            TRY(sys->hs.ensure(rid_mlp_fp32_scratch_floats(E, W) * sizeof(float)));
         } else {
             const size_t ntiles = (size_t)(W + 127) / 128;
             TRY(sys->tsave.ensure((size_t)E.M * ntiles * E.L * 128 * E.H * sizeof(__nv_bfloat16)));
@@ -946,8 +946,8 @@ static int tune_tc_stages(rid_system* sys, TcArgs P, cudaStream_t st) {
     return RID_OK;
 }
 
-// values_only: the member values alone (the tensor-core kernel then runs the
-// L forward GEMMs and skips the input gradient; the FP32 kernel forms both).
+// values_only: the member values alone (the kernels then run the L forward
+// GEMMs and skip the input gradient; the small FP32 kernel forms both).
 static int launch_mlp(rid_system* sys, int W, int mode, StateDev sd, cudaStream_t st, bool values_only) {
     EnsDev& E = sys->E;
     if (mode == 1 && sys->precision != RID_PREC_FP32) {
@@ -1012,7 +1012,7 @@ static int launch_mlp(rid_system* sys, int W, int mode, StateDev sd, cudaStream_
         E.aslices = 1;
     } else if (mode == 1) {
         E.aslices = 1;
-        TRY(timed_launch(sys, "k_mlp_fp32", st, [&] { rid_launch_mlp_fp32(E, sd, W, sys->S.C, st); }));
+        TRY(timed_launch(sys, "k_mlp_fp32", st, [&] { rid_launch_mlp_fp32(E, sd, W, sys->S.C, st, values_only); }));
     }
     return RID_OK;
 }
@@ -1356,7 +1356,7 @@ size_t rid_sys_footprint(const rid_system* sys, int W) {
     if (sys->has_ens) {
         const EnsDev& E = sys->E;
         b += (size_t)E.M * nc * 4 + (size_t)E.M * W * 4;
-        if (sys->precision == RID_PREC_FP32) b += rid_mlp_fp32_scratch_floats(W, E.M, E.L, E.H) * 4;
+        if (sys->precision == RID_PREC_FP32) b += rid_mlp_fp32_scratch_floats(E, W) * 4;
         else b += (size_t)E.M * ((W + 127) / 128) * 128 * (E.H * (E.L * 2 + (E.resnet ? 4 : 0)) + TC_MAX_QSLICES * 4);
     }
     return b;

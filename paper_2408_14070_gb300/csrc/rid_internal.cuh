@@ -285,8 +285,32 @@ void rid_launch_label_final(const LabelDev& lab, int W, int C, double* mf, doubl
                             cudaStream_t s);
 void rid_launch_philox(long long n, const uint32_t* ctr, uint32_t k0, uint32_t k1, uint32_t* words,
                        float* normals, cudaStream_t s);
-void rid_launch_mlp_fp32(const EnsDev& E, StateDev st, int W, int C, cudaStream_t s);
-size_t rid_mlp_fp32_scratch_floats(int W, int M, int L, int H);
+// One FP32 evaluation of an ensemble (k_mlp_fp32): W^T of layer l of member m
+// at WT + m wt_st + toff[l], rows of ldt floats (a multiple of 4, zero past H);
+// W_l [H][fin] at Wb + m wb_st + woff[l] (input gradient only).
+struct MlpF32 {
+    const float* WT;
+    const float* Wb;
+    long long wt_st, wb_st, toff[RID_MAX_LAYERS], woff[RID_MAX_LAYERS];
+    int ldt;
+    const float* b;          // bias of layer l of member m at b + m b_st + boff[l]
+    long long b_st, boff[RID_MAX_LAYERS];
+    const float* wout;
+    const float* bout;
+    long long wo_st, bo_st;
+    const float* u;          // [W][D]
+    int D, L, H, resnet, W, C;
+    float* hs;               // rid_mlp_fp32_scratch_floats (input gradient only)
+    float* Aval;             // [M][W]
+    float* gradA;            // [M][W][C]
+    const int* cvdist;
+};
+// values_only: the member values may be formed without the input gradient
+void rid_launch_mlp_fp32(const EnsDev& E, StateDev st, int W, int C, cudaStream_t s, bool values_only = false);
+size_t rid_mlp_fp32_scratch_floats(const EnsDev& E, int W);
+// Member values alone; split sums the K tiles of 32 with even and odd index apart
+// (the order of MCMC batches below 1024 walkers or 64 columns).
+void rid_launch_mlp_values(const MlpF32& E, int M, bool split, cudaStream_t s);
 // Set the calling thread's rid_last_error message; returns code.
 int rid_fail(int code, const char* fmt, ...);
 // Device description and device ordinal of a system (defined with rid_system).

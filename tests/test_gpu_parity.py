@@ -197,6 +197,32 @@ def test_small_ensembles_on_walker_tiles(R, orc, n, C, W, M, L, H, resnet, seed)
         assert abs(abar[w] - e["Abar"]) <= FORCE_RTOL * (abs(e["Abar"]) + 1.0), w
 
 
+@pytest.mark.parametrize("W,M,C,H,resnet", [
+    (9, 4, 18, 160, False),       # 8-walker tiles, a ragged second one
+    (700, 4, 3, 256, False),      # 32-walker tiles, 6 inputs: rows that are not 16-byte aligned
+    (2000, 4, 7, 200, True),      # 56-walker tiles, a padded width, residual
+    (2300, 4, 20, 256, False),    # 64-walker tiles
+    (333, 2, 128, 512, True),     # four warp columns, the most inputs, residual
+    (70, 1, 5, 288, False),       # four warp columns, the third a quarter full
+])
+def test_fp32_ensemble_on_every_walker_tile(R, orc, W, M, C, H, resnet):
+    """The FP32 ensemble kernel's tile shapes (walkers per CTA by walker count, warp columns by width) against the
+    oracle on walkers of the first, a middle and the last tile."""
+    n, L = max(24, C + 4), 3
+    sp = I.make_system(n, C, 3)
+    x = np.tile(I.make_chains(min(W, 64), sp, 3), (W // min(W, 64) + 1, 1, 1))[:W]
+    x = (x + np.random.default_rng(W).normal(0.0, 0.02, x.shape)).astype(np.float32)
+    ens = I.make_ensemble(M, 2 * C, L, H, 3, resnet=resnet)
+    s, abar, g = np.zeros((W, C), np.float32), np.zeros(W, np.float32), np.zeros((M, W, C), np.float32)
+    with R.System(sp) as sys:
+        sys.set_ensemble(ens)
+        sys.eval_forces(x, R.RID_BIAS_ENSEMBLE, s_out=s, abar_out=abar, grad_out=g)
+    for w in sorted({0, 7, W // 2, W - 2, W - 1}):
+        e = orc.ensemble(ens, orc.cvs(sp, x[w].astype(np.float64))[0])
+        assert close_rel(g[:, w], e["gradA"], FORCE_RTOL) < 1.0, w
+        assert abs(abar[w] - e["Abar"]) <= FORCE_RTOL * (abs(e["Abar"]) + 1.0), w
+
+
 def test_fp32_ensemble_at_the_size_limits(R, orc):
     # 128 torsion CVs (256 MLP inputs) and width 512: the FP32 ensemble
     # kernel's largest shared-memory footprint (activations, inputs and the
