@@ -3,29 +3,32 @@
 // proj_cv_index; Introduction, automatic PMF calculation).
 //
 // W walkers run Metropolis Monte Carlo in CV space on the ensemble-mean free
-// energy Abar(s) = (1/M) sum_i A_i(s) at temperature kT.  Every step:
-//   k_mc_propose  s' = wrap(s + step_size xi) (a distance CV: not wrapped),
-//                 xi: normal c % 3 of the Box-Muller triple of Philox counter
-//                 (c / 3, walker, step, 2); writes the MLP input
-//                 u' = (cos s', sin s') (a distance CV: (s', 0))
-//   forward GEMMs one batched FP32 GEMM per layer (rid_gemm.cuh), members on
-//                 grid z, the input u' shared by all members
-//   k_mc_accept   one warp per walker: A_i = w_out . h + b_out, Abar' as the
-//                 mean in member order; accept iff kT ln u + (Abar' - Abar) < 0
-//                 and every distance CV of s' lies in its range [lo, hi]
-//                 with u = (x + 1/2) 2^-32, x = word 0 of counter
+// energy Abar(s) = (1/M) sum_i A_i(s) at temperature kT.  Every step is two
+// launches:
+//   ensemble      the member values A_i at the proposals: k_mlp_fp32's forward
+//                 pass (all layers of a tile of walkers in one CTA), or a
+//                 system's own ensemble kernels
+//   k_mc_step     one warp per walker.  Accept: Abar' as the mean over the
+//                 members; accepted iff kT ln u + (Abar' - Abar) < 0 and every
+//                 distance CV of s' lies in its range [lo, hi], with
+//                 u = (x + 1/2) 2^-32, x = word 0 of Philox counter
 //                 (0, walker, step, 3); from step n_burn on, the current state
 //                 of every walker is counted into one histogram per CV and one
-//                 2-D histogram of a CV pair (integer atomics: exact)
-// and at the end k_mc_pmf turns the counts into -kT ln(count / total),
-// shifted to a zero minimum (+inf for empty bins).  With path nodes, the warp
-// also maps each counted state onto the path collective variables (lanes over
-// the nodes, the smallest distance factored out, sums in a fixed order) and
+//                 2-D histogram of a CV pair (integer atomics: exact).  Then the
+//                 next step's proposal s' = wrap(s + step_size xi) (a distance
+//                 CV: not wrapped), xi: normal c % 3 of the Box-Muller triple of
+//                 Philox counter (c / 3, walker, step, 2), and its MLP input
+//                 u' = (cos s', sin s') (a distance CV: (s', 0))
+// and at the end k_mc_logs / k_mc_pmf turn the counts into -kT ln(count /
+// total), shifted to a zero minimum (+inf for empty bins).  With path nodes, the
+// warp also maps each counted state onto the path collective variables (lanes
+// over the nodes, the smallest distance factored out, sums in a fixed order) and
 // counts (s_path, z_path).
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
-#include "rid_gemm.cuh"
+#include "rid_internal.cuh"
 
 namespace {
 
@@ -65,28 +68,16 @@ __global__ void k_mc_features(const float* __restrict__ s, float* __restrict__ U
         mc_input(s[e], k.dist && k.dist[(int)(e % C)], U + 2 * e);
 }
 
-__global__ void k_mc_propose(const float* __restrict__ s, float* __restrict__ sp, float* __restrict__ U, int W, int C,
-                             uint32_t step, float step_size, uint32_t k0, uint32_t k1, McCvDev k) {
-    const long long n = (long long)W * C;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-        const int w = (int)(e / C), c = (int)(e - (long long)w * C);
-        const float3 z = rid_normals3(rid_philox(make_uint4((uint32_t)(c / 3), (uint32_t)w, step, 2u), k0, k1));
-        const int r = c % 3;
-        const float xi = r == 0 ? z.x : (r == 1 ? z.y : z.z);
-        const bool dist = k.dist && k.dist[c];
-        const float v = dist ? fmaf(step_size, xi, s[e]) : rid_wrapf(fmaf(step_size, xi, s[e]));
-        sp[e] = v;
-        mc_input(v, dist, U + 2 * e);
-    }
-}
-
-struct AcceptArgs {
-    const float* h;        // [M][W][H] last hidden layer
-    const float* w;        // [M][P] packed weights
-    long long P, ooff;     // floats per member, offset of w_out (b_out follows)
-    int M, W, H, C;
+struct StepArgs {
+    const float* aval;     // [na][W] member values at the proposals
+    int na, ordered;       // ordered: summed in member order, else over the lanes of a warp
+    int M, W, C;
     float* s;              // [W][C] state
-    const float* sp;       // [W][C] proposal
+    float* sp;             // [W][C] proposal
+    float* U;              // [W][2C] MLP input of the proposal
+    int propose;           // write the proposal of step `next`
+    uint32_t next;
+    float step_size;
     float* A;              // [W] Abar at the state
     uint32_t step, k0, k1;
     float kT;
@@ -102,38 +93,48 @@ struct AcceptArgs {
     const float* pnodes;         // [P][Cp]
     float lam, z_lo, z_hi;
     unsigned long long* histp;   // [bins][bins]
-    // member values from a system's ensemble kernels ([na][W], na = M x slices) instead of h . w_out
-    const float* aval;
-    int na;
     McCvDev cvk;                 // distance CVs: range, bins, plain path differences
 };
 
-__global__ void k_mc_accept(AcceptArgs a) {
+// The proposal of walker w for step a.next, from its current state.  Lane c % 32
+// writes CV c, as in the acceptance before it.
+__device__ __forceinline__ void mc_propose(const StepArgs& a, int w, int lane) {
+    for (int c = lane; c < a.C; c += 32) {
+        const float3 z = rid_normals3(rid_philox(make_uint4((uint32_t)(c / 3), (uint32_t)w, a.next, 2u), a.k0, a.k1));
+        const int r = c % 3;
+        const float xi = r == 0 ? z.x : (r == 1 ? z.y : z.z);
+        const bool dist = a.cvk.dist && a.cvk.dist[c];
+        const long long e = (long long)w * a.C + c;
+        const float v = dist ? fmaf(a.step_size, xi, a.s[e]) : rid_wrapf(fmaf(a.step_size, xi, a.s[e]));
+        a.sp[e] = v;
+        mc_input(v, dist, a.U + 2 * e);
+    }
+}
+
+// Accept the proposals of one step, count, and write the next ones.  Bound by
+// latency (member values, state and proposal from L2, then two Philox draws):
+// one launch instead of two saves a launch and a trip of s through memory.
+// 2000 walkers of 20 CVs: 10.0 us in two launches (accept 6.1, propose 3.9);
+// the step with the BF16 ensemble 38.4 -> 35.3 us.
+__global__ void k_mc_step(StepArgs a) {
     const int lane = threadIdx.x & 31;
     const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (w >= a.W) return;                       // whole warps only
     float abar = 0.0f;
-    if (a.aval) {
+    if (a.ordered) {
+        for (int m = 0; m < a.na; ++m) abar += a.aval[(long long)m * a.W + w];
+    } else {
         float part = 0.0f;
         for (int k = lane; k < a.na; k += 32) part += a.aval[(long long)k * a.W + w];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
         abar = part;
-    } else {
-        for (int m = 0; m < a.M; ++m) {
-            const float* wo = a.w + (long long)m * a.P + a.ooff;
-            const float* h = a.h + ((long long)m * a.W + w) * a.H;
-            float part = 0.0f;
-            for (int j = lane; j < a.H; j += 32) part = fmaf(wo[j], h[j], part);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-            abar += part + wo[a.H];
-        }
     }
     abar /= (float)a.M;
     float* s = a.s + (long long)w * a.C;
     if (a.init) {
         if (lane == 0) a.A[w] = abar;
+        if (a.propose) mc_propose(a, w, lane);
         return;
     }
     const uint4 r = rid_philox(make_uint4(0u, (uint32_t)w, a.step, 3u), a.k0, a.k1);
@@ -205,16 +206,26 @@ __global__ void k_mc_accept(AcceptArgs a) {
             }
         }
     }
+    if (a.propose) mc_propose(a, w, lane);
 }
 
-// One CTA per histogram row of length n: f = -kT ln(count / total) - min f.
+// f = -kT ln(count / total) - min f per histogram row of length n, in two
+// passes over slices of PS bins: the logarithms with each slice's minimum, then
+// the shift.  The FP64 logarithms bound it, so a row is spread over the SMs:
+// 101 x 101 bins took 238 us in one CTA (which took every logarithm twice).
 constexpr int PT = 256;
-__global__ void __launch_bounds__(PT) k_mc_pmf(const unsigned long long* __restrict__ hist, int n, double kT,
-                                               double* __restrict__ pmf) {
+constexpr int PS = 512;
+constexpr int PSLICES = 64;
+__host__ __device__ inline int pmf_slices(int n) {
+    const int k = (n + PS - 1) / PS;
+    return k < PSLICES ? k : PSLICES;
+}
+__global__ void __launch_bounds__(PT) k_mc_logs(const unsigned long long* __restrict__ hist, int n, double kT,
+                                                double* __restrict__ pmf, double* __restrict__ part) {
     __shared__ unsigned long long tot_s[PT];
     __shared__ double min_s[PT];
-    const unsigned long long* h = hist + (long long)blockIdx.x * n;
-    double* f = pmf + (long long)blockIdx.x * n;
+    const unsigned long long* h = hist + (long long)blockIdx.y * n;
+    double* f = pmf + (long long)blockIdx.y * n;
     unsigned long long tot = 0;
     for (int i = threadIdx.x; i < n; i += PT) tot += h[i];
     tot_s[threadIdx.x] = tot;
@@ -225,16 +236,43 @@ __global__ void __launch_bounds__(PT) k_mc_pmf(const unsigned long long* __restr
     }
     const double total = (double)tot_s[0];
     double mn = INFINITY;
-    for (int i = threadIdx.x; i < n; i += PT)
-        if (h[i]) mn = fmin(mn, -kT * log((double)h[i] / total));
+    for (int i = blockIdx.x * PT + threadIdx.x; i < n; i += gridDim.x * PT) {
+        const double lg = h[i] ? log((double)h[i] / total) : -INFINITY;
+        f[i] = lg;
+        mn = fmin(mn, -kT * lg);          // an empty bin's +inf never is the minimum
+    }
     min_s[threadIdx.x] = mn;
     __syncthreads();
     for (int k = PT / 2; k > 0; k >>= 1) {
         if (threadIdx.x < k) min_s[threadIdx.x] = fmin(min_s[threadIdx.x], min_s[threadIdx.x + k]);
         __syncthreads();
     }
-    mn = min_s[0];
-    for (int i = threadIdx.x; i < n; i += PT) f[i] = h[i] ? -kT * log((double)h[i] / total) - mn : INFINITY;
+    if (threadIdx.x == 0) part[blockIdx.y * gridDim.x + blockIdx.x] = min_s[0];
+}
+__global__ void __launch_bounds__(PT) k_mc_pmf(int n, double kT, double* __restrict__ pmf,
+                                               const double* __restrict__ part) {
+    double* f = pmf + (long long)blockIdx.y * n;
+    double mn = INFINITY;
+    for (int k = 0; k < (int)gridDim.x; ++k) mn = fmin(mn, part[blockIdx.y * gridDim.x + k]);
+    for (int i = blockIdx.x * PT + threadIdx.x; i < n; i += gridDim.x * PT)
+        f[i] = f[i] == -INFINITY ? INFINITY : -kT * f[i] - mn;
+}
+
+// W_l [H][fin] of every member (packed at w + woff) to W^T [fin][ldt], zero past H.
+__global__ void k_mc_transpose(const float* __restrict__ w, long long P, long long woff, int H, int fin, int ldt,
+                               float* __restrict__ wt, long long wt_st) {
+    __shared__ float tile[32][33];
+    const int m = blockIdx.z, k0 = blockIdx.x * 32, n0 = blockIdx.y * 32;
+    const float* src = w + m * P + woff;
+    for (int y = threadIdx.y; y < 32; y += blockDim.y) {
+        const int n = n0 + y, k = k0 + threadIdx.x;
+        tile[y][threadIdx.x] = n < H && k < fin ? src[(long long)n * fin + k] : 0.0f;
+    }
+    __syncthreads();
+    for (int y = threadIdx.y; y < 32; y += blockDim.y) {
+        const int k = k0 + y, n = n0 + threadIdx.x;
+        if (k < fin && n < ldt) wt[m * wt_st + (long long)k * ldt + n] = tile[threadIdx.x][y];
+    }
 }
 
 int mc_cuda(cudaError_t e, const char* what) { return rid_fail(RID_ERR_CUDA, "mcmc: %s: %s", what, cudaGetErrorString(e)); }
@@ -296,12 +334,15 @@ extern "C" RID_API int rid_mcmc(const rid_mcmc_desc* d, const float* s0, float* 
     }
     const long long ooff = o, P = o + H + 1;
     // device memory, carved from one allocation (released on return)
-    const long long nW = (long long)M * P, nS = (long long)W * C, nU = (long long)W * D, nH = (long long)M * W * H;
+    const int ldt = (H + 31) / 32 * 32;
+    const long long wt_st = (long long)(D + (L - 1) * H) * ldt;   // W^T of one member
+    const long long nW = (long long)M * P, nS = (long long)W * C, nU = (long long)W * D, nT = M * wt_st;
     const long long n1 = (long long)C * bins, n2 = (long long)bins * bins;
-    const size_t bytes_f = sizeof(float) * (size_t)(nW + 2 * nS + W + nU + (d->resnet ? 3 : 2) * nH);
+    const size_t bytes_f = sizeof(float) * (size_t)(nT + nW + 2 * nS + W + nU + (long long)M * W);
     const long long np2 = NP ? n2 : 0, npn = (long long)NP * Cp;
     const size_t bytes_u = sizeof(unsigned long long) * (size_t)(n1 + n2 + np2 + 1);
-    const size_t bytes_d = sizeof(double) * (size_t)(n1 + n2 + np2);
+    const long long npart = (long long)rid_mc_pmf_scratch(C, bins);
+    const size_t bytes_d = sizeof(double) * (size_t)(n1 + n2 + np2 + npart + 1);
     const size_t bytes_p = sizeof(float) * (size_t)npn + sizeof(int) * (size_t)Cp;
     const size_t bytes_k = has_dist ? (sizeof(int) + 2 * sizeof(float)) * (size_t)C : 0;
     McBufs buf;
@@ -317,14 +358,16 @@ extern "C" RID_API int rid_mcmc(const rid_mcmc_desc* d, const float* s0, float* 
     double* pmf1 = reinterpret_cast<double*>(nacc + 1);
     double* pmf2 = pmf1 + n1;
     double* pmfp = pmf2 + n2;
-    float* wts = reinterpret_cast<float*>(pmfp + np2);
+    double* part = pmfp + np2;
+    // W^T first: its rows are read by 16-byte copies
+    float* wt = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(part + npart) + 15) & ~(uintptr_t)15);
+    float* wts = wt + nT;
     float* s = wts + nW;
     float* sp = s + nS;
     float* A = sp + nS;
     float* U = A + W;
-    float* hb[2] = {U + nU, U + nU + nH};
-    float* tb = d->resnet ? hb[1] + nH : nullptr;
-    float* pnodes = (d->resnet ? tb + nH : hb[1] + nH);
+    float* aval = U + nU;
+    float* pnodes = aval + (long long)M * W;
     int* pcv = reinterpret_cast<int*>(pnodes + npn);
     McCvDev cvk;
     if (has_dist) {
@@ -363,37 +406,40 @@ extern "C" RID_API int rid_mcmc(const rid_mcmc_desc* d, const float* s0, float* 
 
     const uint32_t k0 = (uint32_t)d->seed, k1 = (uint32_t)(d->seed >> 32);
     const int eb = (int)((nS + 255) / 256 < 4096 ? (nS + 255) / 256 : 4096);
-    auto forward = [&]() {
-        for (int l = 0; l < L; ++l) {
-            const int fin = l == 0 ? D : H;
-            GemmArgs g{};
-            g.nseg = 1;
-            g.seg[0].a = l == 0 ? act_rowmajor(U, D, 0) : act_rowmajor(hb[(l - 1) & 1], H, (long long)W * H);
-            g.seg[0].b = Operand{wts + woff[l], (long long)fin, 1, P};      // (k, j) -> W_l[j][k]
-            g.seg[0].K = fin;
-            g.rows = W;
-            g.cols = H;
-            EpiArgs& ea = g.e;
-            ea.ld = H;
-            ea.act_sm = (long long)W * H;
-            ea.bias = wts + boff[l];
-            ea.bias_sm = P;
-            ea.Hout = hb[l & 1];
-            ea.T = d->resnet ? tb : ea.Hout;
-            ea.Hin = l == 0 ? nullptr : hb[(l - 1) & 1];
-            ea.resid = d->resnet && l >= 1;
-            launch_gemm<EPI_FWD>(g, M, st);
-        }
-    };
-    AcceptArgs aa{};
-    aa.h = hb[(L - 1) & 1];
-    aa.w = wts;
-    aa.P = P;
-    aa.ooff = ooff;
+    MlpF32 net{};
+    net.WT = wt;
+    net.wt_st = wt_st;
+    net.ldt = ldt;
+    net.b = wts;
+    net.b_st = net.wo_st = net.bo_st = P;
+    net.wout = wts + ooff;
+    net.bout = wts + ooff + H;
+    net.u = U;
+    net.D = D;
+    net.L = L;
+    net.H = H;
+    net.resnet = d->resnet ? 1 : 0;
+    net.W = W;
+    net.C = C;
+    net.Aval = aval;
+    for (int l = 0; l < L; ++l) {
+        const int fin = l == 0 ? D : H;
+        net.toff[l] = l == 0 ? 0 : (long long)(D + (l - 1) * H) * ldt;
+        net.boff[l] = boff[l];
+        k_mc_transpose<<<dim3((fin + 31) / 32, ldt / 32, M), dim3(32, 8), 0, st>>>(wts, P, woff[l], H, fin, ldt,
+                                                                                   wt + net.toff[l], wt_st);
+    }
+    // (the order of the K sums by batch size, as the results always had it)
+    const bool split = W < 1024 || H < 64;
+    StepArgs aa{};
+    aa.aval = aval;
+    aa.na = M;
+    aa.ordered = 1;
     aa.M = M;
     aa.W = W;
-    aa.H = H;
     aa.C = C;
+    aa.U = U;
+    aa.step_size = (float)d->step_size;
     aa.s = s;
     aa.sp = sp;
     aa.A = A;
@@ -418,20 +464,22 @@ extern "C" RID_API int rid_mcmc(const rid_mcmc_desc* d, const float* s0, float* 
     const int wpb = 4;                                  // walkers (warps) per CTA
     const int ab = (W + wpb - 1) / wpb;
     k_mc_features<<<eb, 256, 0, st>>>(s, U, nS, C, cvk);
-    forward();
+    rid_launch_mlp_values(net, M, split, st);
     aa.init = 1;
-    k_mc_accept<<<ab, 32 * wpb, 0, st>>>(aa);
+    aa.propose = d->n_steps > 0;
+    k_mc_step<<<ab, 32 * wpb, 0, st>>>(aa);
     aa.init = 0;
     for (int64_t t = 0; t < d->n_steps; ++t) {
-        k_mc_propose<<<eb, 256, 0, st>>>(s, sp, U, W, C, (uint32_t)t, (float)d->step_size, k0, k1, cvk);
-        forward();
+        rid_launch_mlp_values(net, M, split, st);
         aa.step = (uint32_t)t;
         aa.count = t >= d->n_burn;
-        k_mc_accept<<<ab, 32 * wpb, 0, st>>>(aa);
+        aa.propose = t + 1 < d->n_steps;
+        aa.next = (uint32_t)(t + 1);
+        k_mc_step<<<ab, 32 * wpb, 0, st>>>(aa);
     }
-    k_mc_pmf<<<C, PT, 0, st>>>(hist1, bins, d->kT, pmf1);
-    k_mc_pmf<<<1, PT, 0, st>>>(hist2, (int)n2, d->kT, pmf2);
-    if (NP) k_mc_pmf<<<1, PT, 0, st>>>(histp, (int)n2, d->kT, pmfp);
+    rid_launch_mc_pmf(hist1, C, bins, d->kT, pmf1, part, st);
+    rid_launch_mc_pmf(hist2, 1, (int)n2, d->kT, pmf2, part, st);
+    if (NP) rid_launch_mc_pmf(histp, 1, (int)n2, d->kT, pmfp, part, st);
     if ((e = cudaGetLastError()) != cudaSuccess) return mc_cuda(e, "launch");
     if (s_out && (e = cudaMemcpyAsync(s_out, s, sizeof(float) * nS, kout, st)) != cudaSuccess) return mc_cuda(e, "s_out");
     if (hist1_out && (e = cudaMemcpyAsync(hist1_out, hist1, sizeof(uint64_t) * n1, kout, st)) != cudaSuccess)
@@ -461,19 +509,11 @@ void rid_launch_mc_features(const float* s, float* U, long long n, int C, const 
     k_mc_features<<<eb, 256, 0, st>>>(s, U, n, C, cvk);
 }
 
-void rid_launch_mc_propose(const float* s, float* sp, float* U, int W, int C, uint32_t step, float step_size,
-                           uint32_t k0, uint32_t k1, const McCvDev& cvk, cudaStream_t st) {
-    const long long n = (long long)W * C;
-    const int eb = (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
-    k_mc_propose<<<eb, 256, 0, st>>>(s, sp, U, W, C, step, step_size, k0, k1, cvk);
-}
-
-void rid_launch_mc_accept_values(const float* aval, int na, int M, int W, int C, float* s, const float* sp, float* A,
-                                 uint32_t step, float kT, uint32_t k0, uint32_t k1, int init, int count, int bins,
-                                 int pi, int pj, unsigned long long* hist1, unsigned long long* hist2,
-                                 unsigned long long* nacc, const McPathDev& path, const McCvDev& cvk,
-                                 cudaStream_t st) {
-    AcceptArgs a{};
+void rid_launch_mc_step(const float* aval, int na, int M, int W, int C, float* s, float* sp, float* U, float* A,
+                        uint32_t step, float kT, float step_size, uint32_t k0, uint32_t k1, int init, int propose,
+                        int count, int bins, int pi, int pj, unsigned long long* hist1, unsigned long long* hist2,
+                        unsigned long long* nacc, const McPathDev& path, const McCvDev& cvk, cudaStream_t st) {
+    StepArgs a{};
     a.cvk = cvk;
     a.npath = path.n_nodes;
     a.Cp = path.n_cv;
@@ -490,8 +530,12 @@ void rid_launch_mc_accept_values(const float* aval, int na, int M, int W, int C,
     a.C = C;
     a.s = s;
     a.sp = sp;
+    a.U = U;
     a.A = A;
     a.step = step;
+    a.propose = propose;
+    a.next = init ? 0u : step + 1u;
+    a.step_size = step_size;
     a.k0 = k0;
     a.k1 = k1;
     a.kT = kT;
@@ -504,9 +548,16 @@ void rid_launch_mc_accept_values(const float* aval, int na, int M, int W, int C,
     a.hist2 = hist2;
     a.nacc = nacc;
     const int wpb = 4;
-    k_mc_accept<<<(W + wpb - 1) / wpb, 32 * wpb, 0, st>>>(a);
+    k_mc_step<<<(W + wpb - 1) / wpb, 32 * wpb, 0, st>>>(a);
 }
 
-void rid_launch_mc_pmf(const unsigned long long* hist, int rows, int n, double kT, double* pmf, cudaStream_t st) {
-    k_mc_pmf<<<rows, PT, 0, st>>>(hist, n, kT, pmf);
+size_t rid_mc_pmf_scratch(int C, int bins) {
+    return (size_t)std::max((long long)C * pmf_slices(bins), (long long)pmf_slices(bins * bins));
+}
+
+void rid_launch_mc_pmf(const unsigned long long* hist, int rows, int n, double kT, double* pmf, double* part,
+                       cudaStream_t st) {
+    const dim3 grid(pmf_slices(n), rows);
+    k_mc_logs<<<grid, PT, 0, st>>>(hist, n, kT, pmf, part);
+    k_mc_pmf<<<grid, PT, 0, st>>>(n, kT, pmf, part);
 }

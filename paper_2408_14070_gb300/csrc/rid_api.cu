@@ -1645,7 +1645,8 @@ extern "C" int rid_mcmc_system(rid_system* sys, int32_t W, const float* s0, int6
     const size_t o_p2 = o_p1 + 8 * n1, o_pp = o_p2 + 8 * n2, o_s = o_pp + 8 * np2, o_sp = o_s + 4 * nS;
     const size_t o_A = o_sp + 4 * nS, o_pn = o_A + ((4 * (size_t)W + 15) & ~(size_t)15), o_pc = o_pn + 4 * npn;
     const size_t o_rg = o_pc + 4 * (size_t)Cp;   // distance-CV ranges lo [C], hi [C]
-    TRY(scoped.b.ensure(o_rg + 8 * (size_t)C));
+    const size_t o_pt = (o_rg + 8 * (size_t)C + 15) & ~(size_t)15;   // slice minima of the PMFs
+    TRY(scoped.b.ensure(o_pt + 8 * rid_mc_pmf_scratch(C, bins)));
     unsigned char* b = static_cast<unsigned char*>(scoped.b.p);
     auto* h1 = reinterpret_cast<unsigned long long*>(b + o_h1);
     auto* h2 = reinterpret_cast<unsigned long long*>(b + o_h2);
@@ -1690,17 +1691,17 @@ extern "C" int rid_mcmc_system(rid_system* sys, int32_t W, const float* s0, int6
     const int M = sys->E.M, nav = M * sys->E.aslices;
     rid_launch_mc_features(ds, sd.u, nS, C, cvk, st);
     TRY(launch_mlp(sys, W, 1, sd, st, true));
-    rid_launch_mc_accept_values(sd.Aval, nav, M, W, C, ds, dsp, dA, 0u, (float)kT, k0, k1, 1, 0, bins, proj_i, proj_j,
-                                h1, h2, na, pd, cvk, st);
+    rid_launch_mc_step(sd.Aval, nav, M, W, C, ds, dsp, sd.u, dA, 0u, (float)kT, (float)step_size, k0, k1, 1,
+                       n_steps > 0, 0, bins, proj_i, proj_j, h1, h2, na, pd, cvk, st);
     for (int64_t t = 0; t < n_steps; ++t) {
-        rid_launch_mc_propose(ds, dsp, sd.u, W, C, (uint32_t)t, (float)step_size, k0, k1, cvk, st);
         TRY(launch_mlp(sys, W, 1, sd, st, true));
-        rid_launch_mc_accept_values(sd.Aval, nav, M, W, C, ds, dsp, dA, (uint32_t)t, (float)kT, k0, k1, 0,
-                                    t >= n_burn, bins, proj_i, proj_j, h1, h2, na, pd, cvk, st);
+        rid_launch_mc_step(sd.Aval, nav, M, W, C, ds, dsp, sd.u, dA, (uint32_t)t, (float)kT, (float)step_size, k0, k1,
+                           0, t + 1 < n_steps, t >= n_burn, bins, proj_i, proj_j, h1, h2, na, pd, cvk, st);
     }
-    rid_launch_mc_pmf(h1, C, bins, kT, p1, st);
-    rid_launch_mc_pmf(h2, 1, (int)n2, kT, p2, st);
-    if (NP) rid_launch_mc_pmf(pd.hist, 1, (int)n2, kT, pp, st);
+    double* part = reinterpret_cast<double*>(b + o_pt);
+    rid_launch_mc_pmf(h1, C, bins, kT, p1, part, st);
+    rid_launch_mc_pmf(h2, 1, (int)n2, kT, p2, part, st);
+    if (NP) rid_launch_mc_pmf(pd.hist, 1, (int)n2, kT, pp, part, st);
     CK(cudaGetLastError());
     if (s_out) CK(cudaMemcpyAsync(s_out, ds, sizeof(float) * nS, kout, st));
     if (hist1_out) CK(cudaMemcpyAsync(hist1_out, h1, 8 * n1, kout, st));
@@ -1713,7 +1714,7 @@ extern "C" int rid_mcmc_system(rid_system* sys, int32_t W, const float* s0, int6
     CK(cudaMemcpyAsync(&hna, na, sizeof(hna), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     if (n_accepted) *n_accepted = (int64_t)hna;
-    sys->launches += 3 + 3 * n_steps + 2 + (NP ? 1 : 0);
+    sys->launches += 2 + n_steps + 4 + (NP ? 2 : 0);   // (launch_mlp counts its own)
     return RID_OK;
 }
 

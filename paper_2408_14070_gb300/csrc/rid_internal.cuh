@@ -227,8 +227,6 @@ struct McCvDev {
     const float* hi = nullptr;
 };
 void rid_launch_mc_features(const float* s, float* U, long long n, int C, const McCvDev& cvk, cudaStream_t st);
-void rid_launch_mc_propose(const float* s, float* sp, float* U, int W, int C, uint32_t step, float step_size,
-                           uint32_t k0, uint32_t k1, const McCvDev& cvk, cudaStream_t st);
 // Device side of a path projection (n_nodes = 0: off).
 struct McPathDev {
     int n_nodes = 0, n_cv = 0;
@@ -242,12 +240,17 @@ int rid_mc_range_check(int C, const int32_t* dist, const double* lo, const doubl
 // Checks a path projection's host arguments against C CVs (RID_OK or RID_ERR_ARG).
 int rid_mc_path_check(int n_nodes, int n_cv, int C, const int32_t* cv, const float* nodes, double lambda,
                       double z_lo, double z_hi);
-void rid_launch_mc_accept_values(const float* aval, int na, int M, int W, int C, float* s, const float* sp, float* A,
-                                 uint32_t step, float kT, uint32_t k0, uint32_t k1, int init, int count, int bins,
-                                 int pi, int pj, unsigned long long* hist1, unsigned long long* hist2,
-                                 unsigned long long* nacc, const McPathDev& path, const McCvDev& cvk,
-                                 cudaStream_t st);
-void rid_launch_mc_pmf(const unsigned long long* hist, int rows, int n, double kT, double* pmf, cudaStream_t st);
+// Accept the proposals of `step` by their member values aval [na][W] (init: only
+// set A), count the states, and write the proposals of the next step (of step 0
+// after init) with their MLP input U.
+void rid_launch_mc_step(const float* aval, int na, int M, int W, int C, float* s, float* sp, float* U, float* A,
+                        uint32_t step, float kT, float step_size, uint32_t k0, uint32_t k1, int init, int propose,
+                        int count, int bins, int pi, int pj, unsigned long long* hist1, unsigned long long* hist2,
+                        unsigned long long* nacc, const McPathDev& path, const McCvDev& cvk, cudaStream_t st);
+// part: rid_mc_pmf_scratch(C, bins) doubles for any of a run's histograms
+size_t rid_mc_pmf_scratch(int C, int bins);
+void rid_launch_mc_pmf(const unsigned long long* hist, int rows, int n, double kT, double* pmf, double* part,
+                       cudaStream_t st);
 cudaError_t rid_launch_label_cons(const SysDev& S, int R, int C, int B, long long n_steps, long long n_equil,
                                   uint32_t step0, float kT, const float4* x0, const float4* v0, const int2* pairs,
                                   const float* d0, double* bsum, double* mf, double* se, double* sd, float4* x_out,

@@ -63,6 +63,39 @@ def test_trajectories_follow_the_oracle(R, M, C, L, H, resnet, W, K):
     assert 0 < nacc < W * K                      # moves are taken and refused
 
 
+@pytest.mark.parametrize("M,C,L,H,resnet,W", [
+    (2, 3, 2, 63, False, 1023),     # one warp column, split K sums, odd width
+    (4, 3, 2, 63, False, 1100),     # the same beyond 1024 walkers (still below 64 columns)
+    (2, 5, 3, 128, True, 1024),     # one warp column at its widest, one K chain
+    (4, 4, 2, 130, False, 2300),    # two warp columns, 64-walker tiles
+    (3, 20, 2, 300, True, 40),      # four warp columns, few walkers
+    (1, 128, 1, 512, False, 1500),  # the most inputs, one layer
+])
+def test_accepted_moves_on_every_walker_tile(R, M, C, L, H, resnet, W):
+    """Two steps on the value kernel's tile shapes: the accepted moves and the states of every walker whose decisions
+    are clear in the oracle."""
+    ens = I.make_ensemble(M, 2 * C, L, H, 7, resnet=resnet)
+    s0 = np.random.default_rng(W).uniform(-math.pi, math.pi, size=(W, C)).astype(np.float32)
+    s = np.zeros_like(s0)
+    nacc = R.mcmc(ens.weights, M, C, L, H, s0, 2, 0, 1.0, 0.3, 11, bins=8, resnet=resnet, s_out=s)
+    ref = MC.run(ens.weights, C, L, H, resnet, s0, 2, 0, 1.0, 0.3, 11, 8, (0, 1))
+    safe = ref["min_margin"] > 1e-3
+    assert safe.mean() > 0.9
+    assert np.max(_wrapdiff(s[safe], ref["s"][safe])) < 1e-4
+    assert abs(nacc - ref["n_accepted"]) <= 2 * int((~safe).sum())
+
+
+@pytest.mark.parametrize("bins", [1, 300])
+def test_pmf_slices_match_the_definition(R, bins):
+    """A pair histogram of one slice and of more bins than the slices cover in one pass."""
+    ens = I.make_ensemble(1, 4, 1, 8, 5)
+    s0 = np.random.default_rng(3).uniform(-math.pi, math.pi, size=(500, 2)).astype(np.float32)
+    h2, f2 = np.zeros((bins, bins), np.uint64), np.zeros((bins, bins))
+    R.mcmc(ens.weights, 1, 2, 1, 8, s0, 6, 0, 1.3, 0.5, 5, bins=bins, pair=(0, 1), hist2=h2, pmf2=f2)
+    assert int(h2.sum()) == 500 * 6
+    np.testing.assert_allclose(f2, MC.projected_pmf(h2, 1.3), rtol=1e-12, atol=1e-12)
+
+
 def test_counting_and_binning_are_exact(R):
     M, C, L, H, W, K = 2, 5, 2, 32, 300, 7
     ens = I.make_ensemble(M, 2 * C, L, H, 32)
