@@ -122,6 +122,33 @@ def test_trajectory_follows_the_oracle(R, M, C, L, H, B, n, resnet):
     assert not np.array_equal(w, ens.weights)
 
 
+@pytest.mark.parametrize("M,C,L,H,B,resnet,rate", [
+    (3, 3, 2, 37, 33, True, 0.1),      # odd width: padded rows; one row past a tile
+    (2, 37, 3, 130, 31, False, 0.0),   # 74 inputs, two columns past a tile
+    (1, 128, 1, 512, 40, False, 0.1),  # the most inputs and K, one layer
+    (1, 33, 3, 96, 1025, True, 0.1),   # a large batch: 64-wide tiles, the loss over their pairs
+    (2, 5, 2, 60, 1030, False, 0.0),   # a large batch of fewer than 64 columns: 32-wide tiles
+])
+def test_gradient_on_the_tile_edges(R, M, C, L, H, B, resnet, rate):
+    # (tolerances of the file's head)
+    ens, s, mf, idx = _problem(M, C, L, H, B, 500, 23, resnet)
+    loss = np.zeros(M, np.float32)
+    grad = np.zeros((M, ens.weights.shape[1]), np.float32)
+    kw = dict(dropout_rate=rate, dropout_seed=9) if rate else {}
+    with R.Trainer(M, C, L, H, ens.weights, batch_size=B, resnet=resnet, **kw) as tr:
+        tr.set_data(s, mf)
+        tr.grad(idx, loss, grad)
+        tr.run(idx[None])
+        w, _ = tr.weights()
+    q = T.dropout_scales(M, B, L, H, 0, 9, rate) if rate else [None] * M
+    for m in range(M):
+        lo, go = T.loss_and_grad(ens.weights[m].astype(np.float64), 2 * C, L, H, resnet, s[idx[m]], mf[idx[m]], q[m])
+        assert abs(loss[m] - lo) <= 1e-5 * lo
+        assert np.linalg.norm(grad[m] - go) / np.linalg.norm(go) < 1e-4
+        step = grad[m].astype(np.float64) / (np.abs(grad[m]) + 1e-8)      # Adam's first step: lr g / (|g| + eps)
+        assert np.abs(w[m] - (ens.weights[m] - 8e-4 * step)).max() < 1e-6
+
+
 @pytest.mark.parametrize("rate", [0.1, 0.5])
 @pytest.mark.parametrize("M,C,L,H,B,n,resnet", SHAPES[:2])
 def test_dropout_loss_and_gradient_match_the_oracle(R, M, C, L, H, B, n, resnet, rate):
