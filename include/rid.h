@@ -592,13 +592,12 @@ typedef struct {
 
 /*
  * Batched restrained labeling (Sec. "Labeling phase", restrained method):
- * every run of every job in ONE persistent kernel launch that keeps each
- * chain resident in shared memory for all of its steps.  Jobs may differ in
- * chain length, CV count, restraints and step counts.  Each job's outputs are
- * bit-identical to rid_label on the same inputs.
- *   threads     CTA size of the persistent kernel: 128, 256 or 512, or 0 to
- *               pick it by timing the batch itself for a few steps (the
- *               choice is cached per batch shape on the server)
+ * every run of every job in one persistent kernel launch per class of chain
+ * lengths, the launches side by side, each chain resident in shared memory for
+ * all of its steps.  Jobs may differ in chain length, CV count, restraints and step counts.
+ * Each job's outputs are bit-identical to rid_label on the same inputs.
+ *   threads     CTA size of every run: 128, 256 or 512, or 0 to choose it by
+ *               chain length
  *   status_out  [n_jobs] | NULL: per job RID_OK or RID_ERR_NONFINITE
  * `mem` applies to every array of every job.  Synchronous.  The jobs' device
  * memory comes from the server pool and is released before the call returns.

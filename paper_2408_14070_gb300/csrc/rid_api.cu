@@ -1564,18 +1564,14 @@ extern "C" int rid_label(rid_system* sys, int32_t R, const float* x0, const floa
         A.items = reinterpret_cast<const FusedItem*>(dm + o_items);
         A.n_items = R;
         A.next = reinterpret_cast<int*>(dm + o_cnt);
-        const size_t smem = rid_label_fused_smem(N, C, 0);
-        int nt = N <= 128 ? 128 : (N <= 256 ? 256 : 512);
-        if (rid_label_fused_occupancy(nt, smem) < 1) nt = 128;
-        int occ = rid_label_fused_occupancy(nt, smem);
-        if (occ < 1) return fail(RID_ERR_ARG, "label runs of %d beads exceed shared memory", N);
         int nsm = 1, dev = 0;
         CK(cudaGetDevice(&dev));
         CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-        const int grid = (int)std::min<long long>(R, (long long)occ * nsm);
+        const int nt = rid_label_run_threads(N);
         cudaError_t le = cudaSuccess;
-        TRY(timed_launch(sys, "k_label_fused", st, [&] { le = rid_launch_label_fused(A, nt, grid, smem, st); }));
-        if (le != cudaSuccess) return fail(RID_ERR_CUDA, "k_label_fused launch: %s", cudaGetErrorString(le));
+        TRY(timed_launch(sys, "k_label_run", st,
+                         [&] { le = rid_launch_label_run(A, nt, nsm, rid_label_run_smem(N, C), st); }));
+        if (le != cudaSuccess) return fail(RID_ERR_CUDA, "k_label_run launch: %s", cudaGetErrorString(le));
         // the host staging vector must outlive the copy
         CK(cudaStreamSynchronize(st));
     } else {

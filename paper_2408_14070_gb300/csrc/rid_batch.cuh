@@ -41,6 +41,17 @@ struct FusedArgs {
     int* next;            // work counter, zero at launch
 };
 
+// One CTA per run, the terms of a step as tasks of its warps (k_label_run).
+// Shared memory for N beads and C CVs, 0 when it does not fit (from about 870
+// beads on):
+size_t rid_label_run_smem(int N, int C);
+// CTA size for a chain of N beads: a warp for every task of a step, up to 16.
+// (More runs than fit at once want it too: 512 uneven runs of 50 to 500 beads
+// took 5.5 ms at 512 threads, 6.4 at 256 and 9.6 at 128.)
+int rid_label_run_threads(int N);
+// threads: 128, 256 or 512; smem: the largest over the items.
+cudaError_t rid_launch_label_run(const FusedArgs& A, int threads, int n_sm, size_t smem, cudaStream_t s);
+
 // Dynamic shared memory of k_label_fused for a chain of N beads and C CVs.
 size_t rid_label_fused_smem(int N, int C, int threads);
 // Launch on `s` with `threads` per CTA (128, 256 or 512) and `grid` CTAs;

@@ -250,6 +250,134 @@ __device__ __forceinline__ void lj_row_culled(const SysDev& S, const float4* xs,
     }
 }
 
+// Neighbour lists of a chain that stays in shared memory over many steps.  The
+// list of bead i holds, in increasing j, every j that is not excluded and lies
+// within 1.2 rc when the list is built; as long as no bead has moved more than
+// half of that skin since (0.1 rc), every pair inside the cutoff is in it, and the row
+// sum over the list adds what lj_row_culled adds, in its order, less some pairs
+// that add exactly +0: the same bits for 11 pairs a bead instead of 80 to 200.
+// (In k_ff, whose lists lay in HBM for one step's use, they cost more than they
+// saved.)  Entries nl[k * NP + i] with the count in k = 0, cap at most: a row of
+// 32 beads with a longer list (over[row]) is evaluated by lj_row_culled.
+constexpr float LJ_NEAR2 = 1.44f;            // (list radius / rc)^2
+constexpr float LJ_MOVED2 = 0.0992f * 0.0992f;   // (displacement / rc)^2 that keeps a list valid: just below 0.1
+
+// Build the lists of the warp's 32 beads wlo .. (chains of up to 2048 beads).  A
+// position that is not a number counts as near.
+__device__ __forceinline__ void lj_list_build(const SysDev& S, const float4* xs, const float4* cbox, int nclus, int wlo,
+                                              unsigned short* nl, int NP, int cap, int* over) {
+    const int lane = threadIdx.x & 31, i = wlo + lane, N = S.N;
+    const float rl2 = LJ_NEAR2 * S.rc2;
+    const float3 xi = f3(xs[i < N ? i : N - 1]);
+    // the warp's box: its (up to) four clusters'
+    float3 ilo = make_float3(INFINITY, INFINITY, INFINITY), ihi = make_float3(-INFINITY, -INFINITY, -INFINITY);
+    for (int c = wlo / LJ_CLUSTER; c < min(nclus, wlo / LJ_CLUSTER + 4); ++c) {
+        const float4 lo = cbox[2 * c], hi = cbox[2 * c + 1];
+        ilo = make_float3(fminf(ilo.x, lo.x), fminf(ilo.y, lo.y), fminf(ilo.z, lo.z));
+        ihi = make_float3(fmaxf(ihi.x, hi.x), fmaxf(ihi.y, hi.y), fmaxf(ihi.z, hi.z));
+    }
+    int cnt = 0, g = 0;
+    unsigned mask = 0, ids = 0;       // 8 bits a cluster, 8 bits its number
+    auto drain = [&]() {
+        while (mask) {
+            const int b = __ffs(mask) - 1;
+            mask &= mask - 1;
+            if (++cnt <= cap)
+                nl[cnt * NP + i] = (unsigned short)(LJ_CLUSTER * ((ids >> (b & 24)) & 255u) + (b & 7));
+        }
+        ids = 0;
+        g = 0;
+    };
+    for (int w = 0; w < nclus; w += 32) {
+        bool kp = false;
+        if (w + lane < nclus) {
+            const float4 lo = cbox[2 * (w + lane)], hi = cbox[2 * (w + lane) + 1];
+            const float gx = fmaxf(0.0f, fmaxf(lo.x - ihi.x, ilo.x - hi.x));
+            const float gy = fmaxf(0.0f, fmaxf(lo.y - ihi.y, ilo.y - hi.y));
+            const float gz = fmaxf(0.0f, fmaxf(lo.z - ihi.z, ilo.z - hi.z));
+            kp = !(pair_r2(make_float3(gx, gy, gz)) >= rl2);
+        }
+        for (unsigned m = __ballot_sync(0xffffffffu, kp); m; m &= m - 1) {
+            const int c = w + __ffs(m) - 1;
+            unsigned bits = 0;
+            if (i < N) {
+#pragma unroll
+                for (int k = 0; k < LJ_CLUSTER; ++k) {
+                    const float4 p = xs[LJ_CLUSTER * c + k];
+                    if (!(pair_r2(make_float3(p.x - xi.x, p.y - xi.y, p.z - xi.z)) >= rl2)) bits |= 1u << k;
+                }
+                const int sh = i - 2 - LJ_CLUSTER * c;       // beads i - 2 .. i + 2 are excluded
+                const unsigned ex = sh >= 0 ? (sh < 8 ? 0x1fu << sh : 0u) : (sh > -5 ? 0x1fu >> -sh : 0u);
+                bits &= ~ex;
+            }
+            mask |= bits << (8 * g);
+            ids |= (unsigned)c << (8 * g);
+            if (++g == 4) drain();
+        }
+    }
+    drain();
+    if (i < N) nl[i] = (unsigned short)min(cnt, cap);
+    const bool ov = __any_sync(0xffffffffu, cnt > cap);
+    if (lane == 0) over[wlo >> 5] = ov;
+    __syncwarp();
+}
+
+// Row sums of the warp's 32 beads over their lists.
+template <bool SIG1>
+__device__ __forceinline__ void lj_list_row(const SysDev& S, const float4* xs, const unsigned short* nl, int NP, int i,
+                                            float& fx, float& fy, float& fz) {
+    const float rc2 = S.rc2, sig2 = S.sig2;
+    const bool act = i < S.N;
+    const int cnt = act ? nl[i] : 0;
+    const float3 xi = f3(xs[act ? i : 0]);
+    const int most = __reduce_max_sync(0xffffffffu, cnt);
+    for (int k0 = 1; k0 <= most; k0 += 4) {
+        float c[4];
+        float3 d[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const bool on = k0 + u <= cnt;
+            const float4 p = xs[on ? nl[(k0 + u) * NP + i] : (act ? i : 0)];
+            d[u] = make_float3(p.x - xi.x, p.y - xi.y, p.z - xi.z);
+            const float r2 = pair_r2(d[u]);
+            const float inv = rcp_approx(r2);
+            const float sr2 = SIG1 ? inv : sig2 * inv;
+            const float sr6 = sr2 * sr2 * sr2;
+            c[u] = inv * (sr6 * fmaf(2.0f, sr6, -1.0f));
+            c[u] = on && r2 < rc2 ? c[u] : 0.0f;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            fx = fmaf(c[u], d[u].x, fx);
+            fy = fmaf(c[u], d[u].y, fy);
+            fz = fmaf(c[u], d[u].z, fz);
+        }
+    }
+}
+
+// Bounding box of each aligned group of eight lanes' positions (a cluster), for
+// lanes with act set (the group's first lane always); written by that lane.
+__device__ __forceinline__ void lj_lane_boxes(float3 x, bool act, int i, float4* cbox) {
+    const int first = threadIdx.x & 24;
+    const float3 x0 = make_float3(__shfl_sync(0xffffffffu, x.x, first), __shfl_sync(0xffffffffu, x.y, first),
+                                  __shfl_sync(0xffffffffu, x.z, first));
+    float3 lo = act ? x : x0, hi = lo;
+#pragma unroll
+    for (int o = 1; o < LJ_CLUSTER; o <<= 1) {
+        lo.x = fminf(lo.x, __shfl_xor_sync(0xffffffffu, lo.x, o));
+        lo.y = fminf(lo.y, __shfl_xor_sync(0xffffffffu, lo.y, o));
+        lo.z = fminf(lo.z, __shfl_xor_sync(0xffffffffu, lo.z, o));
+        hi.x = fmaxf(hi.x, __shfl_xor_sync(0xffffffffu, hi.x, o));
+        hi.y = fmaxf(hi.y, __shfl_xor_sync(0xffffffffu, hi.y, o));
+        hi.z = fmaxf(hi.z, __shfl_xor_sync(0xffffffffu, hi.z, o));
+    }
+    if (act && (threadIdx.x & 7) == 0) {
+        const int c = i / LJ_CLUSTER;
+        cbox[2 * c] = make_float4(lo.x, lo.y, lo.z, 0.0f);
+        cbox[2 * c + 1] = make_float4(hi.x, hi.y, hi.z, 0.0f);
+    }
+}
+
 // Bonded force on bead i in the order of bonded_gather: bonds and angles are
 // recomputed here, the dihedral terms come from the shared slots fD written by
 // bonded_dihedrals_to_smem.  Adds are non-contractible, so the result is

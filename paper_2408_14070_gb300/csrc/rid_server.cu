@@ -1,8 +1,8 @@
 // rid_server.cu -- the server object: device memory of a fixed budget
 // (segments allocated on demand, first-fit inside each segment), pinned
 // staging, batched restrained labeling through the persistent kernel
-// k_label_fused (one launch for any number of uneven jobs) with a timing
-// autotuner for its CTA size, and the request loop (rid_submit / rid_poll):
+// kernels of k_label_run.cu (one launch per CTA size, chosen by chain length)
+// and k_label_fused.cu (chains too long for it), and the request loop (rid_submit / rid_poll):
 // a worker thread that admits jobs by device footprint and runs label jobs in
 // ticks of the persistent kernel and exploration jobs as replayed CUDA graphs.
 #include <algorithm>
@@ -288,8 +288,9 @@ struct rid_server {
     Pinned pin_in, pin_out, pin_meta;    // batch call staging
     void* d_meta = nullptr;              // batch call tables (grow-only, outside the budget)
     size_t d_meta_bytes = 0;
-    std::map<long long, int> tuned;      // batch-shape key -> CTA size
-    int last_threads = 0;
+    // a batch's launches, one per CTA size, run side by side
+    cudaStream_t bst[3] = {};
+    cudaEvent_t bfork = nullptr, bjoin[3] = {};
     // request loop
     std::chrono::steady_clock::time_point t0;
     std::mutex mu;                       // queue, job records
@@ -373,13 +374,6 @@ int check_label_job(const rid_label_job& j, int idx, int device) {
     if (!j.sys || !j.x0 || !j.s0 || !j.kappa || !j.mf_out || !j.se_out || !j.std_out)
         return rid_fail(RID_ERR_ARG, "job %d: NULL argument", idx);
     return check_label_args(j.sys, j.n_runs, j.n_blocks, j.step0, j.n_steps, j.n_equil, idx, device);
-}
-
-long long shape_key(int n_items, int maxN) {
-    int a = 0, b = 0;
-    while ((1 << a) < n_items && a < 30) ++a;
-    while ((1 << b) < maxN && b < 30) ++b;
-    return (long long)a * 64 + b;
 }
 
 // Fill the device pointers of a label job placed at `b`.
@@ -607,7 +601,6 @@ int label_tick_launch(rid_server* srv) {
     std::vector<FusedItem> items;
     size_t in_h = 0, out_h = 0;
     double pred = 0.0;
-    int maxN = 0;
     size_t smem = 0, smem_cl = 0;
     for (size_t k = 0; k < act.size(); ++k) {
         SJob* j = act[k];
@@ -623,7 +616,6 @@ int label_tick_launch(rid_server* srv) {
         j->t_next = J.t1;
         fj[k] = J;
         pred = std::max(pred, per * steps);
-        maxN = std::max(maxN, j->N);
         (cl ? smem_cl : smem) = std::max(cl ? smem_cl : smem, rid_label_fused_smem(j->N, j->C, 0));
         for (int r = 0; r < j->W; ++r) items.push_back({(int)k, r});
         if (!j->staged) {
@@ -694,11 +686,6 @@ int label_tick_launch(rid_server* srv) {
     A2.n_items = n_big;
     A2.next = reinterpret_cast<int*>(dm + o_cnt + 128);
     int nt = 256;
-    {
-        std::lock_guard<std::mutex> lk(srv->pool_mu);
-        auto hit = srv->tuned.find(shape_key((int)items.size(), maxN));
-        if (hit != srv->tuned.end()) nt = hit->second;
-    }
     const size_t smem_all = std::max(smem, smem_cl);
     if (rid_label_fused_occupancy(nt, smem_all) < 1) nt = 128;
     SCK(cudaMemsetAsync(A.next, 0, 256, st));
@@ -911,6 +898,11 @@ extern "C" int rid_server_destroy(rid_server* srv) {
     if (srv->lfork) cudaEventDestroy(srv->lfork);
     if (srv->ljoin) cudaEventDestroy(srv->ljoin);
     if (srv->lst2) cudaStreamDestroy(srv->lst2);
+    if (srv->bfork) cudaEventDestroy(srv->bfork);
+    for (int k = 0; k < 3; ++k) {
+        if (srv->bjoin[k]) cudaEventDestroy(srv->bjoin[k]);
+        if (srv->bst[k]) cudaStreamDestroy(srv->bst[k]);
+    }
     delete srv;
     return RID_OK;
 }
@@ -1040,8 +1032,6 @@ extern "C" int rid_label_batch(rid_server* srv, const rid_label_job* jobs, int32
     std::vector<char*> off(n_jobs, nullptr);
     size_t in_bytes = 0, out_bytes = 0;
     std::vector<size_t> in_off(n_jobs), out_off(n_jobs);
-    int maxN = 0;
-    size_t smem = 0;
     long long n_items = 0;
     for (int k = 0; k < n_jobs; ++k) {
         const rid_label_job& j = jobs[k];
@@ -1052,8 +1042,6 @@ extern "C" int rid_label_batch(rid_server* srv, const rid_label_job* jobs, int32
         in_bytes += align_up(12 * nb * (j.v0 ? 2 : 1) + 16 * nc);
         out_off[k] = out_bytes;
         out_bytes += align_up(24 * nc + 4 * (size_t)j.n_runs + 12 * nb * ((j.x_out ? 1 : 0) + (j.v_out ? 1 : 0)));
-        maxN = std::max(maxN, S->N);
-        smem = std::max(smem, rid_label_fused_smem(S->N, S->C, 0));
         n_items += j.n_runs;
     }
     if (n_items > (1 << 30)) return rid_fail(RID_ERR_ARG, "too many runs in one batch");
@@ -1159,6 +1147,30 @@ extern "C" int rid_label_batch(rid_server* srv, const rid_label_job* jobs, int32
         const double cb = (double)jobs[b.job].n_steps * fj[b.job].S.N * fj[b.job].S.N;
         return ca > cb;
     });
+    // one launch per class of runs, so that a short chain does not ask for a long
+    // one's shared memory: classes 0..2 run k_label_run (chains of which one, two,
+    // or more fit an SM), class 3 k_label_fused (chains too long for it)
+    struct Class {
+        int nt = 0, first = 0, n = 0;
+        size_t smem = 0;
+    } cls[4];
+    {
+        auto class_of = [&](const FusedItem& a) {
+            const SysDev& S = fj[a.job].S;
+            const size_t b = rid_label_run_smem(S.N, S.C);
+            return !b ? 3 : b > 112 * 1024 ? 0 : b > 56 * 1024 ? 1 : 2;
+        };
+        std::stable_sort(items.begin(), items.end(),
+                         [&](const FusedItem& a, const FusedItem& b) { return class_of(a) < class_of(b); });
+        for (size_t k = 0; k < items.size(); ++k) {
+            Class& q = cls[class_of(items[k])];
+            const SysDev& S = fj[items[k].job].S;
+            const size_t b = rid_label_run_smem(S.N, S.C);
+            if (!q.n++) q.first = (int)k;
+            q.smem = std::max(q.smem, b ? b : rid_label_fused_smem(S.N, S.C, 0));
+            q.nt = threads ? threads : std::max(q.nt, b ? rid_label_run_threads(S.N) : 512);
+        }
+    }
     // flag copies for the device path go to a small pinned area instead
     std::vector<CopyDesc> dflags;
     if (!host)
@@ -1170,7 +1182,7 @@ extern "C" int rid_label_batch(rid_server* srv, const rid_label_job* jobs, int32
     const size_t o_din = align_up(o_items + sizeof(FusedItem) * items.size());
     const size_t o_dout = align_up(o_din + sizeof(CopyDesc) * din.size());
     const size_t o_cnt = align_up(o_dout + sizeof(CopyDesc) * (dout.size() + dflags.size()));
-    const size_t o_flags = align_up(o_cnt + 16);
+    const size_t o_flags = align_up(o_cnt + 4 * 64);   // a work counter per class
     size_t n_flag_words = 0;
     for (int k = 0; k < n_jobs; ++k) n_flag_words += (size_t)fj[k].R;
     const size_t meta_bytes = align_up(o_flags + 4 * n_flag_words);
@@ -1222,68 +1234,49 @@ extern "C" int rid_label_batch(rid_server* srv, const rid_label_job* jobs, int32
     int rc = [&]() -> int {
         SCK(cudaMemcpyAsync(dm, hm, o_cnt, cudaMemcpyHostToDevice, st));
         if (host) SCK(cudaMemcpyAsync(stage_in, srv->pin_in.p, in_bytes, cudaMemcpyHostToDevice, st));
-        FusedArgs A{};
-        A.jobs = reinterpret_cast<const FusedJob*>(dm + o_jobs);
-        A.items = reinterpret_cast<const FusedItem*>(dm + o_items);
-        A.n_items = (int)items.size();
-        A.next = reinterpret_cast<int*>(dm + o_cnt);
-        const CopyDesc* d_in = reinterpret_cast<const CopyDesc*>(dm + o_din);
-        auto stage = [&]() -> int {
-            rid_launch_copy_descs(d_in, (int)din.size(), st);
-            SCK(cudaGetLastError());
-            return RID_OK;
-        };
-        auto run = [&](int nt) -> int {
-            const int occ = rid_label_fused_occupancy(nt, smem);
-            if (occ < 1) return rid_fail(RID_ERR_CUDA, "k_label_fused<%d> cannot be resident with %zu bytes of shared memory", nt, smem);
-            const int grid = (int)std::min<long long>(n_items, (long long)occ * srv->n_sm);
-            SCK(cudaMemsetAsync(A.next, 0, sizeof(int), st));
-            SCK(rid_launch_label_fused(A, nt, grid, smem, st));
-            return RID_OK;
-        };
-        int nt = threads;
-        const long long key = shape_key((int)n_items, maxN);
-        if (nt == 0) {
-            auto hit = srv->tuned.find(key);
-            if (hit != srv->tuned.end()) nt = hit->second;
-        }
-        if (nt == 0) {
-            // time a short prefix of the batch itself with each CTA size
-            std::vector<FusedJob> trial = fj;
-            long long tmin = 1ll << 60;
-            for (const auto& J : trial) tmin = std::min(tmin, J.n_steps);
-            const long long ts = std::min<long long>(8, tmin);
-            for (auto& J : trial) J.t1 = ts;
-            memcpy(hm + o_jobs, trial.data(), sizeof(FusedJob) * n_jobs);
-            SCK(cudaMemcpyAsync(dm + o_jobs, hm + o_jobs, sizeof(FusedJob) * n_jobs, cudaMemcpyHostToDevice, st));
-            cudaEvent_t e0, e1;
-            SCK(cudaEventCreate(&e0));
-            SCK(cudaEventCreate(&e1));
-            float best = 1e30f;
-            for (int cand : {128, 256, 512}) {
-                if (rid_label_fused_occupancy(cand, smem) < 1) continue;
-                STRY(stage());
-                SCK(cudaEventRecord(e0, st));
-                STRY(run(cand));
-                SCK(cudaEventRecord(e1, st));
-                SCK(cudaEventSynchronize(e1));
-                float ms = 0.f;
-                SCK(cudaEventElapsedTime(&ms, e0, e1));
-                if (ms < best) {
-                    best = ms;
-                    nt = cand;
-                }
+        SCK(cudaMemsetAsync(dm + o_cnt, 0, 4 * 64, st));
+        rid_launch_copy_descs(reinterpret_cast<const CopyDesc*>(dm + o_din), (int)din.size(), st);
+        SCK(cudaGetLastError());
+        int used = 0;
+        for (const Class& c : cls) used += c.n > 0;
+        if (used > 1 && !srv->bfork) {
+            for (int k = 0; k < 3; ++k) {
+                if (!srv->bst[k]) SCK(cudaStreamCreateWithFlags(&srv->bst[k], cudaStreamNonBlocking));
+                if (!srv->bjoin[k]) SCK(cudaEventCreateWithFlags(&srv->bjoin[k], cudaEventDisableTiming));
             }
-            cudaEventDestroy(e0);
-            cudaEventDestroy(e1);
-            if (nt == 0) return rid_fail(RID_ERR_CUDA, "no CTA size of k_label_fused fits %zu bytes of shared memory", smem);
-            srv->tuned[key] = nt;
-            memcpy(hm + o_jobs, fj.data(), sizeof(FusedJob) * n_jobs);
-            SCK(cudaMemcpyAsync(dm + o_jobs, hm + o_jobs, sizeof(FusedJob) * n_jobs, cudaMemcpyHostToDevice, st));
+            SCK(cudaEventCreateWithFlags(&srv->bfork, cudaEventDisableTiming));
         }
-        srv->last_threads = nt;
-        STRY(stage());
-        STRY(run(nt));
+        if (used > 1) SCK(cudaEventRecord(srv->bfork, st));
+        // the largest CTAs first; the last class on the caller's stream
+        int k = 0;
+        for (int c = 0; c < 4; ++c) {
+            if (!cls[c].n) continue;
+            const bool side = k < used - 1;
+            cudaStream_t cst = side ? srv->bst[k] : st;
+            if (side) SCK(cudaStreamWaitEvent(cst, srv->bfork, 0));
+            FusedArgs A{};
+            A.jobs = reinterpret_cast<const FusedJob*>(dm + o_jobs);
+            A.items = reinterpret_cast<const FusedItem*>(dm + o_items) + cls[c].first;
+            A.n_items = cls[c].n;
+            A.next = reinterpret_cast<int*>(dm + o_cnt + 64 * c);
+            if (c < 3) {
+                SCK(rid_launch_label_run(A, cls[c].nt, srv->n_sm, cls[c].smem, cst));
+            } else {
+                int nt = cls[c].nt;
+                while (nt > 128 && rid_label_fused_occupancy(nt, cls[c].smem) < 1) nt /= 2;
+                const int occ = rid_label_fused_occupancy(nt, cls[c].smem);
+                if (occ < 1)
+                    return rid_fail(RID_ERR_CUDA, "k_label_fused<%d> cannot be resident with %zu bytes of shared memory", nt,
+                                    cls[c].smem);
+                SCK(rid_launch_label_fused(A, nt, (int)std::min<long long>(A.n_items, (long long)occ * srv->n_sm),
+                                           cls[c].smem, cst));
+            }
+            if (side) {
+                SCK(cudaEventRecord(srv->bjoin[k], cst));
+                SCK(cudaStreamWaitEvent(st, srv->bjoin[k], 0));
+            }
+            ++k;
+        }
         rid_launch_copy_descs(reinterpret_cast<const CopyDesc*>(dm + o_dout), (int)(dout.size() + dflags.size()), st);
         SCK(cudaGetLastError());
         if (host) SCK(cudaMemcpyAsync(srv->pin_out.p, stage_out, out_bytes, cudaMemcpyDeviceToHost, st));
@@ -1292,6 +1285,8 @@ extern "C" int rid_label_batch(rid_server* srv, const rid_label_job* jobs, int32
         return RID_OK;
     }();
     if (rc != RID_OK) {
+        for (cudaStream_t q : srv->bst)
+            if (q) cudaStreamSynchronize(q);   // a launch made before the failure
         cudaStreamSynchronize(st);
         release();
         return rc;

@@ -67,6 +67,29 @@ def test_batch_is_bit_identical_to_per_job_label(R, threads):
         j["system"].close()
 
 
+@pytest.mark.parametrize("n,C,runs", [
+    (4, 1, 3),          # the shortest chain
+    (64, 30, 2),        # a full half CTA: no thread without a bonded term, CVs on the same threads
+    (65, 3, 2),         # one bead past it
+    (512, 40, 1),       # the longest chain of one LJ pass
+    (513, 5, 1),        # two passes
+    (700, 3, 330),      # more runs than fit at once: smaller CTAs, several runs each
+])
+def test_every_run_shape_gives_the_bits_of_the_per_step_kernels(R, n, C, runs):
+    j = make_job(R, n, C, runs, 24 if runs < 100 else 6, 40 + n, blocks=3)
+    big = make_job(R, 1030, 4, 1, 24, 77, blocks=3)      # beyond the shared bonded slots, beside them
+    with R.Server(1 << 30) as srv:
+        srv.label_batch([j, big])
+    one = alone(j)                                       # rid_label: the same kernel, another CTA size
+    j["system"].set_fused_steps(False)
+    ref = alone(j)                                       # the per-step kernels
+    for k in ("mf", "se", "std", "x_out", "v_out"):
+        assert np.array_equal(j[k], ref[k]), k
+        assert np.array_equal(one[k], ref[k]), k
+    j["system"].close()
+    big["system"].close()
+
+
 def test_batch_on_device_pointers_matches_host(R):
     import torch
     jobs = uneven_jobs(R)[:3]
