@@ -1762,7 +1762,8 @@ extern "C" int rid_label_constrained(rid_system* sys, int32_t R, const float* x0
     } scoped;
     DevBuf& buf = scoped.b;
     const size_t o_x = 0, o_v = o_x + 16 * nb, o_xo = o_v + 16 * nb, o_vo = o_xo + 16 * nb, o_io = o_vo + 16 * nb;
-    const size_t o_bs = o_io + 12 * nb, o_mf = o_bs + 8 * nc * n_blocks, o_se = o_mf + 8 * nc, o_sd = o_se + 8 * nc;
+    // (an odd count of beads would leave the doubles behind the float triples on a 4-byte boundary)
+    const size_t o_bs = o_io + ((12 * nb + 15) & ~15ll), o_mf = o_bs + 8 * nc * n_blocks, o_se = o_mf + 8 * nc, o_sd = o_se + 8 * nc;
     const size_t o_d0 = o_sd + 8 * nc, o_pr = o_d0 + ((4 * nc + 15) & ~15ll), o_bad = o_pr + ((8 * C + 15) & ~15);
     TRY(buf.ensure(o_bad + 4 * R));
     unsigned char* b = static_cast<unsigned char*>(buf.p);

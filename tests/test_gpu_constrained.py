@@ -92,6 +92,20 @@ def test_short_trajectory_follows_the_oracle(R, orc):
     assert np.max(np.abs(r - d0) / d0) < 1e-5
 
 
+def test_odd_number_of_beads_in_all(R, orc):
+    """Three runs of 33 beads: the device buffer of the sums lies behind 99 float triples."""
+    runs = 3
+    sp = I.make_system(33, 2, 5)
+    x0 = I.make_chains(runs, sp, 5)
+    pairs = np.array([[3, 9]], np.int32)
+    d0 = np.ascontiguousarray(np.linalg.norm(x0[:, [3]] - x0[:, [9]], axis=-1), dtype=np.float64)
+    mf, se, sd = (np.zeros((runs, 1)) for _ in range(3))
+    with R.System(sp) as s:
+        s.label_constrained(x0, pairs, d0, 20, 0, 2, mf, se, sd, v0=np.zeros_like(x0))
+    ref = orc.label_constrained(sp, x0, pairs, d0, 20, 0, 2, v0=np.zeros_like(x0))
+    np.testing.assert_allclose(mf, ref["mf"], rtol=1e-3, atol=1e-3)
+
+
 def test_labels_within_standard_errors_of_the_oracle(R, orc):
     runs = 6
     sp, x0, pairs, d0 = _chain_problem(runs, seed=7)
