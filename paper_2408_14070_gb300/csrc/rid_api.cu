@@ -93,8 +93,9 @@ struct TcVariant {
     int gN[2 * RID_MAX_LAYERS] = {0}, gKp[2 * RID_MAX_LAYERS] = {0}, geb[2 * RID_MAX_LAYERS] = {0};
     DevBuf blob, wscale;
     CUtensorMap big{}, small{};
-    // cluster variant (k_mlp_tc_cluster): each GEMM's output columns split over
-    // csize = 2 or 4 CTAs; index 1 = two CTAs, 2 = four.  The cluster size in use
+    // cluster variant (k_mlp_tc_cluster, size 4): each GEMM's output columns split over
+    // csize = 2 or 4 CTAs; index 1 = two CTAs (which sizes rid_set_mlp_cluster takes;
+    // k_mlp_tc_pair runs), 2 = four.  The cluster size in use
     // is chosen by timing the force evaluation at each new walker count.
     bool cl_ok[3] = {false, false, false};
     int cl_stages[3] = {0, 0, 0}, cl_acc_cols[3] = {0, 0, 0}, cl_tmem_cols[3] = {0, 0, 0};
@@ -235,7 +236,7 @@ static int ensure_state(rid_system* sys, int W) {
         if (sys->precision == RID_PREC_FP32) {
             TRY(sys->hs.ensure(rid_mlp_fp32_scratch_floats(E, W) * sizeof(float)));
         } else {
-            const size_t ntiles = (size_t)(W + 127) / 128;
+            const size_t ntiles = rid_tc_tiles(W);
             TRY(sys->tsave.ensure((size_t)E.M * ntiles * E.L * 128 * E.H * sizeof(__nv_bfloat16)));
             if (E.resnet) TRY(sys->rsave.ensure((size_t)E.M * ntiles * 128 * E.H * sizeof(float)));
             TRY(sys->qsave.ensure((size_t)E.M * ntiles * TC_MAX_QSLICES * 128 * sizeof(float)));
@@ -826,29 +827,36 @@ static int launch_forces(rid_system* sys, int W, int mode, bool energy, cudaStre
     return RID_OK;
 }
 
-// The one-CTA ensemble kernel: chunk-interleaved epilogue when the TMEM
-// accumulator is double buffered (width <= 256), the contiguous-column
-// epilogue of k_mlp_tc_wide when a single accumulator fills TMEM.
+// The ensemble kernel of cluster size 1, by size alone.  Two tiles of 128
+// walkers or more: CTA pairs of 128 rows, each CTA with a tile of its own.  One
+// tile: one CTA per member up to width 256, where a pair would take two SMs for
+// the same 39 us (4 x 40-256x4-1); beyond, where the pair's deeper weight
+// stream pays, a pair of 64 rows (8 x 64-512x4-1 at 128 walkers 99 -> 70 us).
+// Measured alone, one CTA per tile -> pairs: 512 wide 120 -> 86 us (2048
+// walkers), 256 wide 39 -> 39 us (1024) and 79 -> 74 us (8192), residual
+// 4 x 36-300x4-1 93 -> 86 us (4096); the same time beside the force field.
+static bool tc1_is_single(const TcArgs& P, const TcVariant& V) { return P.ntiles == 1 && V.nacc == 2; }
 static cudaError_t launch_tc1(const TcArgs& P, const TcVariant& V, cudaStream_t st) {
-    return V.nacc == 1 ? rid_launch_mlp_tc_wide(P, V.big, V.small, st) : rid_launch_mlp_tc(P, V.big, V.small, st);
+    if (tc1_is_single(P, V)) return rid_launch_mlp_tc(P, V.big, V.small, st);
+    return rid_launch_mlp_tc_pair(P, P.ntiles == 1 ? 64 : 128, V.big, V.small, st);
 }
 
-// Cluster size used before the tuner has timed a walker count: the largest
-// of 4 and 2 whose grid (tiles x members x size) still fits the 152 SMs once,
-// else 1 (k_mlp_tc, one CTA per tile and member).
-static int default_cluster(const TcVariant& V, int ctas) {
-    if (V.cl_ok[2] && ctas * 4 <= 152) return 4;
-    if (V.cl_ok[1] && ctas * 2 <= 152) return 2;
-    return 1;
-}
+// Cluster size used before the tuner has timed a walker count, and where
+// nothing runs beside the ensemble: a pair of CTAs per tile (64 rows each)
+// while all pairs fit the 152 SMs at once, else one CTA per tile.  Per launch,
+// one CTA -> pairs of 64: 39 -> 32 us (4 x 40-256x4-1, 1024 walkers), 84 -> 57
+// us (the residual 4 x 36-300x4-1); with twice the SMs' worth of tiles 41 -> 61.
+static int default_cluster(int ctas) { return ctas * 2 <= 152 ? 2 : 1; }
 
 // Autotuner of the ensemble kernel's cluster size: at the first ensemble
 // force evaluation with a new walker count, the whole concurrent phase (the
 // ensemble kernel on the caller's stream, the force field beside it) is timed
-// with each eligible cluster size (1, 2, 4; one warm-up and three timed
-// evaluations each) and the fastest is kept.  Splitting the columns over more
-// CTAs shortens the ensemble's chain but takes SMs from the force field, so
-// the choice is made on the phase, not on the ensemble kernel alone.  Every
+// with cluster sizes 1 and 2 (one warm-up and three timed evaluations, twice
+// in turn) and 2 is kept where it is faster by 8%.  A tile on two CTAs shortens the ensemble's chain but
+// takes SMs from the force field, so the choice is made on the phase, not on
+// the ensemble kernel alone.  (Size 4, k_mlp_tc_cluster, was slower than size 2
+// alone and beside the force field at every size measured: it runs when
+// rid_set_mlp_cluster asks for it.)  Every
 // candidate computes the same quantities; the outputs of the last evaluation
 // are the ones left in place.  Skipped while the stream is being captured.
 static int tune_cluster(rid_system* sys, int W, bool energy, cudaStream_t st) {
@@ -856,16 +864,14 @@ static int tune_cluster(rid_system* sys, int W, bool energy, cudaStream_t st) {
     const int ctas = (W + 127) / 128 * sys->E.M;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     CK(cudaStreamIsCapturing(st, &cs));
-    std::vector<int> cand = {1};
-    if (V.cl_ok[1]) cand.push_back(2);
-    if (V.cl_ok[2]) cand.push_back(4);
     if (sys->serving) {
         V.csize = 1;
         V.cs_W = W;
         return RID_OK;
     }
-    if (cs != cudaStreamCaptureStatusNone || cand.size() == 1) {
-        V.csize = cs != cudaStreamCaptureStatusNone ? default_cluster(V, ctas) : 1;
+    // twice the tiles' CTAs on more than the SMs at once is slower without timing it
+    if (cs != cudaStreamCaptureStatusNone || default_cluster(ctas) == 1) {
+        V.csize = default_cluster(ctas);
         V.cs_W = W;
         return RID_OK;
     }
@@ -873,9 +879,9 @@ static int tune_cluster(rid_system* sys, int W, bool energy, cudaStream_t st) {
     cudaEvent_t a = nullptr, b = nullptr;
     CK(cudaEventCreate(&a));
     CK(cudaEventCreate(&b));
-    float best = 1e30f;
-    int pick = 1;
-    for (int c : cand) {
+    float best[3] = {0.f, 1e30f, 1e30f};
+    for (int k = 0; k < 4; ++k) {
+        const int c = 1 + k % 2;
         V.csize = c;
         V.cs_W = W;
         int rc = launch_forces(sys, W, 1, energy, st);
@@ -893,11 +899,12 @@ static int tune_cluster(rid_system* sys, int W, bool energy, cudaStream_t st) {
         CK(cudaEventSynchronize(b));
         float ms = 0.f;
         CK(cudaEventElapsedTime(&ms, a, b));
-        if (ms < best) {
-            best = ms;
-            pick = c;
-        }
+        best[c] = std::min(best[c], ms);
     }
+    // In a step k_head lies between the evaluations and the force field of a call that fills the SMs
+    // cannot trail into the next one: at 4 x 40-256x4-1 and 1024 x 200 beads, 52 and 50 us here are
+    // 50.3 and 56.4 us a step; where the step gains (41 of 48 us at 100 beads), 15% or more here.
+    const int pick = best[2] < 0.92f * best[1] ? 2 : 1;
     cudaEventDestroy(a);
     cudaEventDestroy(b);
     sys->tuning = false;
@@ -989,22 +996,24 @@ static int launch_mlp(rid_system* sys, int W, int mode, StateDev sd, cudaStream_
             E.aslices = 1;
             return RID_OK;
         }
-        const int cs = sys->cs_force ? sys->cs_force : V.cs_W == W ? V.csize : default_cluster(V, P.ntiles * E.M);
-        if (cs > 1 && !V.cl_ok[cs == 2 ? 1 : 2])
+        const int cs = sys->cs_force ? sys->cs_force : V.cs_W == W ? V.csize : default_cluster(P.ntiles * E.M);
+        if (sys->cs_force > 1 && !V.cl_ok[cs == 2 ? 1 : 2])
             return fail(RID_ERR_ARG, "ensemble kernel: cluster size %d does not fit this ensemble's shape", cs);
         sys->tcv.used_cs = cs;
         if (cs == 1) {
-            if (V.tuned_W != W) TRY(tune_tc_stages(sys, P, st));
+            if (V.tuned_W != W && tc1_is_single(P, V)) TRY(tune_tc_stages(sys, P, st));
             P.stages = V.stages;
             P.csize = 1;
             TRY(timed_launch(sys, "k_mlp_tc", st, [&] { le = launch_tc1(P, V, st); }));
+        } else if (cs == 2) {
+            P.csize = 2;
+            TRY(timed_launch(sys, "k_mlp_tc", st, [&] { le = rid_launch_mlp_tc_pair(P, 64, V.big, V.small, st); }));
         } else {
-            const int k = cs == 2 ? 1 : 2;
             P.csize = cs;
-            P.stages = V.cl_stages[k];
-            P.stage_bytes = V.cl_stage_bytes[k];
-            P.acc_cols = V.cl_acc_cols[k];
-            P.tmem_cols = V.cl_tmem_cols[k];
+            P.stages = V.cl_stages[2];
+            P.stage_bytes = V.cl_stage_bytes[2];
+            P.acc_cols = V.cl_acc_cols[2];
+            P.tmem_cols = V.cl_tmem_cols[2];
             P.nacc = 2;
             TRY(timed_launch(sys, "k_mlp_tc", st, [&] { le = rid_launch_mlp_tc_cluster(P, V.big, V.small, st); }));
         }
@@ -1357,7 +1366,7 @@ size_t rid_sys_footprint(const rid_system* sys, int W) {
         const EnsDev& E = sys->E;
         b += (size_t)E.M * nc * 4 + (size_t)E.M * W * 4;
         if (sys->precision == RID_PREC_FP32) b += rid_mlp_fp32_scratch_floats(E, W) * 4;
-        else b += (size_t)E.M * ((W + 127) / 128) * 128 * (E.H * (E.L * 2 + (E.resnet ? 4 : 0)) + TC_MAX_QSLICES * 4);
+        else b += (size_t)E.M * rid_tc_tiles(W) * 128 * (E.H * (E.L * 2 + (E.resnet ? 4 : 0)) + TC_MAX_QSLICES * 4);
     }
     return b;
 }

@@ -11,6 +11,9 @@
 #define TC_MAX_KCHUNKS 8   // 128-byte K-chunks of the widest GEMM (K <= 512 BF16)
 #define TC_MAX_QSLICES 32  // 16-column slices of the widest hidden layer (512)
 
+// Tiles of 128 walkers in the scratch buffers: whole pairs of them, for the kernel whose CTAs come in pairs.
+inline size_t rid_tc_tiles(int W) { return ((size_t)W + 255) / 256 * 2; }
+
 // Weight image, per member: for GEMM g (forward layers 0..L-1, then backward
 // layers L-1..0) and K-chunk c (128 bytes of K: 64 BF16 or 128 FP8 e4m3
 // columns), the B operand rows [0, N_g) x that column range as rows of 128
@@ -46,8 +49,9 @@ struct TcArgs {
 
 size_t rid_mlp_tc_smem_bytes(const TcArgs& P);
 cudaError_t rid_launch_mlp_tc(const TcArgs& P, const CUtensorMap& big, const CUtensorMap& small, cudaStream_t s);
-size_t rid_mlp_tc_wide_smem_bytes(const TcArgs& P);
-cudaError_t rid_launch_mlp_tc_wide(const TcArgs& P, const CUtensorMap& big, const CUtensorMap& small, cudaStream_t s);
+// CTA pairs (cta_group::2), rows (128 or 64) walkers per CTA; chooses its own weight stages and TMEM columns
+cudaError_t rid_launch_mlp_tc_pair(const TcArgs& P, int rows, const CUtensorMap& big, const CUtensorMap& small,
+                                   cudaStream_t s);
 // Small walker counts (up to 16: NW = 16 MMA columns), BF16, forward and
 // input gradient: the GEMMs transposed (outputs on the MMA's M = 128 rows,
 // walkers on its N columns), each GEMM's 128-output tiles split over a cluster

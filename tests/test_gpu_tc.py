@@ -307,6 +307,48 @@ def test_cluster_sizes_give_identical_bits(R, orc, prec, n, C, W, M, L, H, resne
             assert abs(abar[w] - e["Abar"]) <= tol * (abs(e["Abar"]) + 0.1), w
 
 
+@pytest.mark.parametrize("prec", ["bf16", "fp8"])
+@pytest.mark.parametrize("W,M,L,H,C,resnet", [
+    (129, 2, 3, 256, 5, False),     # one row in the second tile
+    (300, 3, 2, 288, 4, True),      # three tiles (a pair with an empty one), a second block of 32 columns
+    (385, 2, 2, 32, 64, False),     # one 32-column block; the input gradient is the widest GEMM
+    (260, 1, 4, 512, 6, True),      # both blocks full, the residual stream beyond TMEM in rows of 128
+    (1300, 8, 1, 224, 3, True),     # one layer, more tiles than SMs
+])
+def test_tiles_in_pairs_give_the_bits_of_single_tiles(R, orc, prec, W, M, L, H, C, resnet):
+    """A walker's member gradients do not depend on the kernel that its call takes: pairs of 128-row tiles, one tile
+    alone (one CTA, or a pair of 64 rows beyond width 256).  BF16: the oracle's within the bound."""
+    n, seed = max(24, C + 4), 41
+    sp = I.make_system(n, C, seed)
+    x = np.concatenate([I.make_chains(130, sp, seed)] * (W // 130 + 1))[:W].copy()
+    x += np.random.default_rng(seed).normal(0, 0.02, x.shape).astype(np.float32)
+    ens = I.make_ensemble(M, 2 * C, L, H, seed, resnet=resnet, trust_lo=1e9, trust_hi=2e9)
+    p = R.RID_PREC_BF16 if prec == "bf16" else R.RID_PREC_FP8
+    with R.System(sp) as sysobj:
+        sysobj.set_ensemble(ens, precision=p)
+        sysobj.set_mlp_cluster(1)
+
+        def evaluate(part):
+            g = np.zeros((M, len(part), C), np.float32)
+            a = np.zeros(len(part), np.float32)
+            sysobj.eval_forces(part, R.RID_BIAS_ENSEMBLE, abar_out=a, grad_out=g)
+            return g, a
+
+        g, a = evaluate(x)
+        for lo in range(0, W - 17, 250):
+            g1, a1 = evaluate(np.ascontiguousarray(x[lo:lo + 100]))
+            assert np.array_equal(g[:, lo:lo + 100], g1) and np.array_equal(a[lo:lo + 100], a1), lo
+        if 2 * M * -(-W // 128) <= 152:                # the size that a call takes while its pairs fit the SMs
+            sysobj.set_mlp_cluster(0)
+            g2, a2 = evaluate(x)
+            assert np.array_equal(g, g2) and np.array_equal(a, a2)
+    if prec == "bf16":
+        for w in (0, 127, 128, W - 1):
+            e = orc.ensemble(ens, orc.cvs(sp, x[w].astype(np.float64))[0])
+            for m in range(M):
+                assert normwise(g[m, w], e["gradA"][m]) < GRAD_TOL, (w, m)
+
+
 def test_cluster_size_argument_errors(R):
     sp = I.make_system(22, 2, 1)
     with R.System(sp) as sysobj:
