@@ -17,6 +17,16 @@
 // distance (thermodynamic integration with the r^2 Jacobian of the shell):
 //   F_j = dU/dr - 2 kT / d0 = -(f_a - f_b) . u / 2 - 2 kT / d0,
 // summed in FP64 with block sums for the standard error.
+//
+// Forces (LISTS: chains of up to RID_BONDED_SMEM_MAX beads): warps take the LJ
+// rows of 32 beads over neighbour lists kept in shared memory and rebuilt when a
+// bead has moved half the skin, and the bonded terms of 32 beads, each once into
+// per-term slots; then every bead gathers its own.  Bound by issue: at 200 beads
+// a run's step without lists was 10 of 19 thousand instructions of pairs outside
+// the cutoff and angles evaluated by each of their beads.  The same sums in the
+// same order (skipped pairs add exactly zero), so the same bits.
+// 1024 runs x 50 steps of 200 beads: 2.38 -> 1.70 ms (two CTAs of 91 registers an
+// SM before, four now).
 #include "rid_forces.cuh"
 
 namespace {
@@ -42,7 +52,8 @@ struct ConsArgs {
 
 struct ConsLayout {
     int N8, nclus;
-    size_t xs, xo, vs, fs, cbox, fD, sum, sum2, bp, bytes;
+    int NP, cap;                           // LISTS: beads of a list row, longest list
+    size_t xs, xo, vs, fs, cbox, fD, sum, sum2, bp, fB, fA, xr, over, nl, bytes;
 };
 
 __host__ __device__ inline ConsLayout cons_layout(int N, int C) {
@@ -64,7 +75,105 @@ __host__ __device__ inline ConsLayout cons_layout(int N, int C) {
     return L;
 }
 
+// The layout with neighbour lists and all bonded slots (N up to RID_BONDED_SMEM_MAX).  The pre-step
+// positions share the slots' space: those are written and read inside one force evaluation.
+constexpr int CONS_SMEM_MAX = 225 * 1024;
+__host__ __device__ inline ConsLayout cons_layout_lists(int N, int C) {
+    ConsLayout L{};
+    L.nclus = (N + LJ_CLUSTER - 1) / LJ_CLUSTER;
+    L.N8 = L.nclus * LJ_CLUSTER;
+    size_t o = 0;
+    L.xs = o;   o += 16 * (size_t)L.N8;
+    L.vs = o;   o += 16 * (size_t)N;
+    L.fs = o;   o += 16 * (size_t)N;
+    L.cbox = o; o += 32 * (size_t)L.nclus;
+    L.sum = o;  o += 8 * (size_t)C;
+    L.sum2 = o; o += 8 * (size_t)C;
+    L.bp = o;   o += 8 * (size_t)C;
+    o = (o + 15) & ~(size_t)15;
+    L.xo = o;                              // [N] float4, over fD
+    L.fD = o;   o += 48 * (size_t)N;
+    L.fA = o;   o += 36 * (size_t)N;
+    L.fB = o;   o += 12 * (size_t)N;
+    L.xr = o;   o += 12 * (size_t)N;
+    L.over = o; o += 4 * (size_t)((N + 31) / 32);
+    L.NP = (N + 1) / 2 * 2;
+    // 48 entries (a row of 32 beads with a longer list is evaluated without): four runs of 200 beads
+    // an SM; the longest chains keep what there is room for, 16 at least
+    L.nl = o;
+    const size_t room = o < (size_t)CONS_SMEM_MAX ? ((size_t)CONS_SMEM_MAX - o) / (2 * (size_t)L.NP) : 0;
+    L.cap = room > 49 ? 48 : room > 17 ? (int)room - 1 : 16;
+    o += 2 * (size_t)L.NP * (L.cap + 1);
+    L.bytes = (o + 15) & ~(size_t)15;
+    return L;
+}
+
 constexpr int CT = 256;
+
+// Force field of every bead at xs -> fs, over the neighbour lists.  The caller's loop over a thread's
+// beads may follow without a barrier.  first: there are no lists yet.
+__device__ void cons_forces_lists(const SysDev& S, const ConsLayout& L, unsigned char* smem,
+                                  unsigned (*keep_s)[LJ_MAX_MASK_WORDS], bool first, int& bad) {
+    float4* xs = reinterpret_cast<float4*>(smem + L.xs);
+    float4* fs = reinterpret_cast<float4*>(smem + L.fs);
+    float4* cbox = reinterpret_cast<float4*>(smem + L.cbox);
+    float3* fB = reinterpret_cast<float3*>(smem + L.fB);
+    float3* fA = reinterpret_cast<float3*>(smem + L.fA);
+    float3* fD = reinterpret_cast<float3*>(smem + L.fD);
+    float3* xr = reinterpret_cast<float3*>(smem + L.xr);
+    int* over = reinterpret_cast<int*>(smem + L.over);
+    unsigned short* nl = reinterpret_cast<unsigned short*>(smem + L.nl);
+    const int N = S.N, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nb = (N + 31) / 32;
+    const bool sig1 = S.sig2 == 1.0f;
+    const float lj_s = -S.lj_eps24;
+    int moved = first;
+    for (int w0 = 32 * warp; w0 < N; w0 += CT) {
+        const int i = w0 + lane;
+        const float3 x = f3(xs[i < N ? i : N - 1]);
+        if (i < N && !moved) {
+            const float3 d = x - xr[i];
+            moved = !(dot3(d, d) <= LJ_MOVED2 * S.rc2);
+        }
+        lj_lane_boxes(x, i < N, i, cbox);
+    }
+    const int build = __syncthreads_or(moved);
+    for (int k = warp; k < 2 * nb; k += CT / 32) {
+        if (k >= nb) {
+            const int t = 32 * (k - nb) + lane;
+            if (t < N) bonded_terms_to_smem(S, xs, t, fB, fA, fD);
+            continue;
+        }
+        const int i = 32 * k + lane;
+        float fx = 0.f, fy = 0.f, fz = 0.f;
+        if (build) {
+            lj_list_build(S, xs, cbox, L.nclus, 32 * k, nl, L.NP, L.cap, over);
+            if (i < N) xr[i] = f3(xs[i]);
+        }
+        if (over[k]) {
+            float el = 0.f;
+            const float3 xi = f3(xs[i < N ? i : N - 1]);
+            lj_warp_keep_masks(S, cbox, L.nclus, xi, keep_s[warp]);
+            const int b0 = max(32 * k - 2, 0) / LJ_CLUSTER, b1 = min(32 * k + 33, N - 1) / LJ_CLUSTER;
+            const int nwords = (L.nclus + 31) / 32;
+            if (sig1) lj_row_culled<true, false, true>(S, xs, cbox, keep_s[warp], nwords, xi, i, b0, b1, fx, fy, fz, el);
+            else lj_row_culled<false, false, true>(S, xs, cbox, keep_s[warp], nwords, xi, i, b0, b1, fx, fy, fz, el);
+            __syncwarp();
+        } else if (sig1) {
+            lj_list_row<true>(S, xs, nl, L.NP, i, fx, fy, fz);
+        } else {
+            lj_list_row<false>(S, xs, nl, L.NP, i, fx, fy, fz);
+        }
+        if (i < N) fs[i] = make_float4(fx, fy, fz, 0.0f);
+    }
+    __syncthreads();
+    for (int i = tid; i < N; i += CT) {
+        const float3 fb = bonded_gather(S, i, fB, fA, fD);
+        const float4 lj = fs[i];
+        const float4 f = make_float4(fmaf(lj_s, lj.x, fb.x), fmaf(lj_s, lj.y, fb.y), fmaf(lj_s, lj.z, fb.z), 0.0f);
+        bad |= !(isfinite(f.x) && isfinite(f.y) && isfinite(f.z));
+        fs[i] = f;
+    }
+}
 
 // Force field (bonded + culled LJ) of every bead at xs -> fs.
 __device__ void cons_forces(const SysDev& S, float4* xs, float4* cbox, float3* fD, float4* fs,
@@ -143,12 +252,13 @@ __device__ void cons_shake(const int2* pr, int C, const float* d0, const float4*
     }
 }
 
-__global__ void __launch_bounds__(CT) k_label_cons(ConsArgs A) {
+template <bool LISTS>
+__global__ void __launch_bounds__(CT, LISTS ? 4 : 1) k_label_cons(ConsArgs A) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned keep_s[CT / 32][LJ_MAX_MASK_WORDS];
     const SysDev& S = A.S;
     const int N = S.N, C = A.C, r = blockIdx.x, tid = threadIdx.x;
-    const ConsLayout L = cons_layout(N, C);
+    const ConsLayout L = LISTS ? cons_layout_lists(N, C) : cons_layout(N, C);
     float4* xs = reinterpret_cast<float4*>(smem + L.xs);
     float4* xo = reinterpret_cast<float4*>(smem + L.xo);
     float4* vs = reinterpret_cast<float4*>(smem + L.vs);
@@ -196,7 +306,11 @@ __global__ void __launch_bounds__(CT) k_label_cons(ConsArgs A) {
     __syncthreads();
     cons_project_v(A.pairs, C, xs, vs);
     __syncthreads();
-    cons_forces(S, xs, cbox, fD, fs, keep_s, bsm, L.nclus, bad);
+    auto forces = [&](bool first) {
+        if (LISTS) cons_forces_lists(S, L, smem, keep_s, first, bad);
+        else cons_forces(S, xs, cbox, fD, fs, keep_s, bsm, L.nclus, bad);
+    };
+    forces(true);
 
     const long long K = A.n_steps - A.n_equil;
     int cur_b = 0;
@@ -243,7 +357,7 @@ __global__ void __launch_bounds__(CT) k_label_cons(ConsArgs A) {
             __syncthreads();
         }
         half_drift();                                                         // A
-        cons_forces(S, xs, cbox, fD, fs, keep_s, bsm, L.nclus, bad);
+        forces(false);
         half_kick();                                                          // B
         if (t >= A.n_equil) {
             const long long k = t - A.n_equil;
@@ -297,10 +411,13 @@ cudaError_t rid_launch_label_cons(const SysDev& S, int R, int C, int B, long lon
                                   uint32_t step0, float kT, const float4* x0, const float4* v0, const int2* pairs,
                                   const float* d0, double* bsum, double* mf, double* se, double* sd, float4* x_out,
                                   float4* v_out, int* bad, cudaStream_t st) {
-    const size_t smem = rid_label_cons_smem(S.N, C);
-    cudaError_t e = cudaFuncSetAttribute(k_label_cons, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t with_lists = S.N <= RID_BONDED_SMEM_MAX ? cons_layout_lists(S.N, C).bytes : 0;
+    const bool lists = with_lists && with_lists <= (size_t)CONS_SMEM_MAX;
+    const size_t smem = lists ? with_lists : rid_label_cons_smem(S.N, C);
+    const auto kern = lists ? k_label_cons<true> : k_label_cons<false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     ConsArgs A{S, R, C, B, n_steps, n_equil, step0, kT, x0, v0, pairs, d0, bsum, mf, se, sd, x_out, v_out, bad};
-    k_label_cons<<<R, CT, smem, st>>>(A);
+    kern<<<R, CT, smem, st>>>(A);
     return cudaGetLastError();
 }

@@ -106,6 +106,39 @@ def test_odd_number_of_beads_in_all(R, orc):
     np.testing.assert_allclose(mf, ref["mf"], rtol=1e-3, atol=1e-3)
 
 
+@pytest.mark.parametrize("n,runs", [
+    (20, 1),        # one row of 32 beads, partly filled
+    (33, 3),        # one bead in the second row
+    (512, 2),       # more neighbours than a list holds
+    (1024, 1),      # the longest chain with lists
+    (1030, 1),      # beyond: cluster boxes alone
+])
+def test_dense_chains_follow_the_oracle_while_beads_change_neighbours(R, orc, n, runs):
+    """Chains folded on a lattice (80 lattice points within the list radius), thermal velocities: within 20 steps some
+    beads move by more than the lists allow.  Bonds and pairs only (a straight chain's angles and dihedrals are
+    singular).  The bound is the short trajectory's."""
+    sp = I.make_system(n, 2, 3, angle_k=0.0)
+    sp.dihedral_k[:] = 0.0
+    rng = np.random.default_rng(n)
+    side = int(np.ceil(n ** (1 / 3)))
+    k = np.arange(n)
+    z, y, x = k // side ** 2, k // side % side, k % side
+    y = np.where(z % 2, side - 1 - y, y)
+    x = np.where((z * side + k // side % side) % 2, side - 1 - x, x)
+    x0 = (1.15 * np.stack([x, y, z], -1) + rng.uniform(-0.05, 0.05, (runs, n, 3))).astype(np.float32)
+    v0 = rng.standard_normal(x0.shape).astype(np.float32)
+    pairs = np.array([[0, 5], [6, 11], [n - 8, n - 3]], np.int32)
+    d0 = np.ascontiguousarray(np.linalg.norm(x0[:, pairs[:, 0]] - x0[:, pairs[:, 1]], axis=-1), dtype=np.float64)
+    mf, se, sd = (np.zeros((runs, 3)) for _ in range(3))
+    xo, vo = np.zeros_like(x0), np.zeros_like(x0)
+    with R.System(sp) as s:
+        s.label_constrained(x0, pairs, d0, 20, 0, 2, mf, se, sd, v0=v0, x_out=xo, v_out=vo)
+    ref = orc.label_constrained(sp, x0, pairs, d0, 20, 0, 2, v0=v0)
+    assert np.max(np.abs(xo - ref["x"])) < 1e-4
+    assert np.max(np.abs(vo - ref["v"])) < 1e-3
+    np.testing.assert_allclose(mf, ref["mf"], rtol=1e-3, atol=1e-3)
+
+
 def test_labels_within_standard_errors_of_the_oracle(R, orc):
     runs = 6
     sp, x0, pairs, d0 = _chain_problem(runs, seed=7)
