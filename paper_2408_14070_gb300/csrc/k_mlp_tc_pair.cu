@@ -201,6 +201,21 @@ __device__ __forceinline__ void pair_store8(unsigned char* A, int row, int col, 
                                   (uint32_t)((ch ^ (row & 7)) << 4) + (uint32_t)(col & 8)) = pack8_e4m3(v);
     }
 }
+// member_value with its loads ahead of the sums (one latency, not one for every few slices).
+__device__ __forceinline__ float pair_member_value(const TcArgs& P, int m, int tile, int row) {
+    const float* q = P.qsave + qs_off(m, tile, 0, row, P.ntiles);
+    const int n = P.H / 16;
+    float a = 0.0f, v[16];
+    for (int s = 0; s < n; s += 16) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = s + i < n ? q[(s + i) * 128] : 0.0f;
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+            if (s + i < n) a += v[i];
+    }
+    return a + __ldg(P.bout + m);
+}
+
 // 18 warps spread 5/5/4/4 over the four schedulers, each with 16K registers:
 // at most 96 registers per thread
 // F8: the forward GEMMs take FP8 e4m3 operands (the input-gradient GEMMs
@@ -241,19 +256,56 @@ __global__ void __maxnreg__(96)
         S.abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    __syncthreads();
+    __syncwarp();
     cluster_sync_all();               // both CTAs run and their barriers are initialised
-    if (warp == 1) {
+    // TMEM is allocated while the epilogue warps stage the input and the biases and warp 0 starts the weights.
+    // (The even CTA's MMAs wait for arrivals that the odd CTA makes after its own allocation.)
+    float* sbias = reinterpret_cast<float*>(stages + (size_t)NS * PAIR_STAGE);   // [L][H]
+    float* swout = sbias + (size_t)L * P.H;                                      // [H]
+    constexpr int NSUB = ROWS == 128 ? 4 : 8;          // epilogue warps that share a row's columns
+    const int quarter = warp & 3;                      // TMEM lane quarter an epilogue warp may access
+    const int sub = (warp - EPI_WARP0) >> 2;           // its part of the quarter's columns
+    const int hf = ROWS == 128 ? 0 : quarter >> 1;                        // half of each block's columns
+    const int arow = (ROWS == 128 ? quarter : quarter & 1) * 32 + lane;   // row of this CTA's A tile
+    const int subx = ROWS == 128 ? sub : 2 * sub + hf;
+    const int row = row0 + arow;                       // row of the scratch tile
+    const int wg = tile * 128 + row;                   // global walker
+    const bool valid = wg < P.W;
+    if (warp >= EPI_WARP0) {
+        // GEMM 0 input: u (FP32, [W][D], D even) -> its operand format (zeros past D)
+        const int eb0 = F8 ? P.geb[0] : 2;
+        for (int col = 8 * subx; col < P.gKp[0]; col += 8 * NSUB) {
+            float v[8];
+#pragma unroll
+            for (int i = 0; i < 8; i += 2) {
+                float2 q = make_float2(0.0f, 0.0f);
+                if (valid && col + i < P.D)
+                    q = __ldg(reinterpret_cast<const float2*>(P.u + (size_t)wg * P.D + col + i));
+                v[i] = q.x;
+                v[i + 1] = q.y;
+            }
+            pair_store8<ROWS>(Abuf, arow, col, eb0, pack8(v), v);
+        }
+        // biases [L][H], then w_out [H] (H a multiple of 32)
+        const int nb4 = L * P.H / 4;
+        const float4* gb = reinterpret_cast<const float4*>(P.bias + (size_t)m * L * P.H);
+        const float4* gw = reinterpret_cast<const float4*>(P.wout + (size_t)m * P.H);
+        for (int i = threadIdx.x - 32 * EPI_WARP0; i < nb4 + P.H / 4; i += 32 * EPI_WARPS)
+            reinterpret_cast<float4*>(sbias)[i] = i < nb4 ? __ldg(gb + i) : __ldg(gw + i - nb4);
+        fence_async_smem();
+    } else if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&S.tmem_base)),
                      "r"((uint32_t)P.tmem_cols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
-    fence_before();
-    __syncthreads();
-    cluster_sync_all();
-    fence_after();
-    const uint32_t tmem = S.tmem_base;
+    uint32_t tmem = 0;
+    if (warp > 0) {
+        fence_before();
+        asm volatile("bar.sync 1, %0;" ::"r"(NTHREADS - 32) : "memory");
+        fence_after();
+        tmem = S.tmem_base;
+    }
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
@@ -262,6 +314,7 @@ __global__ void __maxnreg__(96)
             int last_it[TC_MAX_STAGES];
             for (int s = 0; s < NS; ++s) last_it[s] = -1;
             bool ok = true;
+            // (N is a multiple of 32: both CTAs load part of every stage, so neither runs ahead of the other)
             for (int g = 0; g < G && ok; ++g) {
                 const int N = P.gN[g], nch = P.gKp[g] * (F8 ? P.geb[g] : 2) / 128;
                 for (int n0 = 0; n0 < N && ok; n0 += 256) {
@@ -348,46 +401,10 @@ __global__ void __maxnreg__(96)
         // ------------------------------------------------------------ epilogue
         // Warp w reads TMEM lane quarter w mod 4 and owns a contiguous quarter
         // (sub = (w - 2) / 4) of the 16-column groups that the quarter's lanes hold.
-        const int e = warp - EPI_WARP0;          // 0..15
-        const int quarter = warp & 3;            // TMEM lane quarter this warp may access
-        const int sub = e >> 2;
-        const int hf = ROWS == 128 ? 0 : quarter >> 1;                 // half of each block's columns
-        const int arow = (ROWS == 128 ? quarter : quarter & 1) * 32 + lane;   // row of this CTA's A tile
-        const int row = row0 + arow;             // row of the scratch tile
-        const int wg = tile * 128 + row;         // global walker
-        const bool valid = wg < P.W;
         const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16);
         const int H = P.H;
-        const int ET = 32 * EPI_WARPS;
-        constexpr int NSUB = ROWS == 128 ? 4 : 8;          // warps that share a row's columns
-        const int subx = ROWS == 128 ? sub : 2 * sub + hf;
         const uint32_t a_bar = smem_u32(&S.a_full);
-        // GEMM 0 input: u (FP32, [W][D], D even) -> its operand format (zeros past D)
-        {
-            const int eb0 = F8 ? P.geb[0] : 2;
-            for (int col = 8 * subx; col < P.gKp[0]; col += 8 * NSUB) {
-                float v[8];
-#pragma unroll
-                for (int i = 0; i < 8; i += 2) {
-                    float2 q = make_float2(0.0f, 0.0f);
-                    if (valid && col + i < P.D)
-                        q = __ldg(reinterpret_cast<const float2*>(P.u + (size_t)wg * P.D + col + i));
-                    v[i] = q.x;
-                    v[i + 1] = q.y;
-                }
-                pair_store8<ROWS>(Abuf, arow, col, eb0, pack8(v), v);
-            }
-            fence_async_smem();
-            __syncwarp();
-            if (lane == 0) pair_arrive(a_bar);
-        }
-        float* sbias = reinterpret_cast<float*>(stages + (size_t)NS * PAIR_STAGE);   // [L][H]
-        float* swout = sbias + (size_t)L * H;                                        // [H]
-        for (int idx = e * 32 + lane; idx < (L + 1) * H; idx += ET) {
-            const int l = idx / H, c = idx - l * H;
-            sbias[idx] = l < L ? __ldg(P.bias + ((size_t)m * L + l) * H + c) : __ldg(P.wout + (size_t)m * H + c);
-        }
-        asm volatile("bar.sync 1, %0;" ::"r"(ET) : "memory");   // all epilogue warps, before any bounded wait
+        if (lane == 0) pair_arrive(a_bar);       // the input is in place
         __nv_bfloat16* tsave_tile = P.tsave + ((size_t)m * P.ntiles + tile) * (size_t)L * 128 * H;
         // residual stream of a resnet ensemble: h_l (forward) and dA/dh_l (backward)
         // in FP32, one [H/8][128][8] block per tile and member, overwritten in place
@@ -591,10 +608,8 @@ __global__ void __maxnreg__(96)
     __syncthreads();
     // member value A = w_out . h_L + b_out: the 16-column partials in column order
     if (warp >= EPI_WARP0 && warp < EPI_WARP0 + 4) {
-        const int arow = (warp & 3) * 32 + lane;
-        const int wg = tile * 128 + row0 + arow;
-        if (arow < ROWS && wg < P.W && !S.abort_flag)
-            P.Apart[(size_t)m * P.W + wg] = member_value(P, m, tile, row0 + arow);
+        if ((ROWS == 128 || hf == 0) && valid && !S.abort_flag)
+            P.Apart[(size_t)m * P.W + wg] = pair_member_value(P, m, tile, row);
     }
     __syncwarp();
     cluster_sync_all();               // no CTA leaves while the pair's MMAs or loads may touch it
