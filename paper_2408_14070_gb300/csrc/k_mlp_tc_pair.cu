@@ -22,9 +22,13 @@
 // even CTA is an arrive without cluster-scope ordering: with it every GEMM
 // waited for the saved activations to reach L2 (4 us of 47 a launch).
 // Measured per launch, one CTA per 128 walkers before -> pairs of 128 rows:
-// 8 x 64-512x4-1 at 8192 walkers 436 -> 319 us, 4 x 40-256x4-1 at 8192 walkers
-// 79 -> 74 us, residual 127 -> 94 us.  What is left is the chain: MMAs and
-// epilogue of one tile alternate (31% tensor time at 512 columns).
+// 8 x 64-512x4-1 at 8192 walkers 436 -> 315 us (682 of 1873 TFLOP/s), 4 x
+// 40-256x4-1 at 8192 walkers 79 -> 73 us, residual 127 -> 94 us; pairs of 64 rows,
+// 1024 walkers of 4 x 40-256x4-1, 39 -> 31 us.  What is left is the chain.  Of 86 us
+// for one wave at 512 columns (2048 walkers), 75 remain without the MMAs, 59 without
+// the epilogue, 38 without both and the weights: hand-overs, saves and the call's
+// ends.  Measured and not kept: the second 256 columns' MMAs under the first's
+// epilogue, its results parked in TMEM (319 -> 310 us, and 5% slower to 256 columns).
 #include "rid_tc_ptx.cuh"
 
 namespace {
@@ -40,7 +44,11 @@ struct Smem {
 };
 
 constexpr uint32_t PAIR_STAGE = 128u * 128u;   // half of a 256-row weight chunk
-constexpr int PAIR_SMEM_MIN = 116 * 1024;      // one CTA per SM, so that a pair never waits for another's TMEM
+// A pair must not hold one SM's TMEM while its other half waits for columns that a CTA of another cluster
+// holds, whose own half may wait for the first SM's.  So the columns of what can share an SM add up to 512 at
+// most: one pair's CTA per SM, and with more than 256 columns nothing else that uses TMEM (no kernel that does
+// fits beside PAIR_SMEM_MAX).
+constexpr size_t PAIR_SMEM_MIN = 116 * 1024, PAIR_SMEM_MAX = 225 * 1024;
 
 __device__ __forceinline__ void pair_mma(bool f8, uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
     if (f8)
@@ -626,17 +634,17 @@ cudaError_t launch_pair(TcArgs P, const CUtensorMap& big, const CUtensorMap& sma
     for (int g = 0; g < P.ngemm; ++g) nmax = P.gN[g] > nmax ? P.gN[g] : nmax;
     // shared memory: the A tile, the biases, and as many weight stages as fit
     const size_t fixed = 1024 + (size_t)P.Kpmax * (2 * ROWS) + sizeof(float) * (size_t)(P.L + 1) * P.H;
-    const size_t budget = 225u * 1024u;
-    if (fixed + 2 * PAIR_STAGE > budget) return cudaErrorInvalidValue;
-    P.stages = (int)((budget - fixed) / PAIR_STAGE);
+    if (fixed + 2 * PAIR_STAGE > PAIR_SMEM_MAX) return cudaErrorInvalidValue;
+    P.stages = (int)((PAIR_SMEM_MAX - fixed) / PAIR_STAGE);
     if (P.stages > TC_MAX_STAGES) P.stages = TC_MAX_STAGES;
     size_t smem = fixed + (size_t)P.stages * PAIR_STAGE;
-    if (smem < PAIR_SMEM_MIN) smem = PAIR_SMEM_MIN;
     // TMEM: the accumulator and, if it fits, a residual network's stream
     P.acc_cols = ROWS == 128 ? nmax : nmax <= 256 ? nmax / 2 : 128 + (nmax - 256) / 2;
     const int cols = P.resnet && P.acc_cols <= 256 ? 2 * P.acc_cols : P.acc_cols;
     P.tmem_cols = 32;
     while (P.tmem_cols < cols) P.tmem_cols *= 2;
+    if (P.tmem_cols > 256) smem = PAIR_SMEM_MAX;
+    else if (smem < PAIR_SMEM_MIN) smem = PAIR_SMEM_MIN;
     if (ROWS == 128) P.ntiles = (P.ntiles + 1) / 2 * 2;   // the scratch buffers hold whole pairs of tiles
     const int v = (P.geb[0] == 1 ? 1 : 0) + (P.resnet ? 2 : 0);
     static size_t attr[4][64] = {};   // shared memory opted into, per instantiation and device

@@ -844,7 +844,7 @@ static cudaError_t launch_tc1(const TcArgs& P, const TcVariant& V, cudaStream_t 
 // Cluster size used before the tuner has timed a walker count, and where
 // nothing runs beside the ensemble: a pair of CTAs per tile (64 rows each)
 // while all pairs fit the 152 SMs at once, else one CTA per tile.  Per launch,
-// one CTA -> pairs of 64: 39 -> 32 us (4 x 40-256x4-1, 1024 walkers), 84 -> 57
+// one CTA -> pairs of 64: 39 -> 31 us (4 x 40-256x4-1, 1024 walkers), 84 -> 57
 // us (the residual 4 x 36-300x4-1); with twice the SMs' worth of tiles 41 -> 61.
 static int default_cluster(int ctas) { return ctas * 2 <= 152 ? 2 : 1; }
 
