@@ -459,11 +459,8 @@ cudaError_t rid_launch_explore_small(const SysDev& S, StateDev st, const EnsDev&
     A.cv_out = cv_out;
     A.eps_out = eps_out;
     const bool bsm = S.N <= RID_BONDED_SMEM_MAX;
-    static unsigned long long attr = 0;
-    if (rid_first_on_device(attr)) {
-        cudaFuncSetAttribute(k_explore_small<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        cudaFuncSetAttribute(k_explore_small<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    }
+    static RidOnce once;
+    if (const cudaError_t e = rid_opt_in(once, 200 * 1024, k_explore_small<true>, k_explore_small<false>)) return e;
     if (bsm) k_explore_small<true><<<W, XS_THREADS, smem, s>>>(A);
     else k_explore_small<false><<<W, XS_THREADS, smem, s>>>(A);
     return cudaGetLastError();

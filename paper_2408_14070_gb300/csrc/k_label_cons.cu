@@ -415,8 +415,8 @@ cudaError_t rid_launch_label_cons(const SysDev& S, int R, int C, int B, long lon
     const bool lists = with_lists && with_lists <= (size_t)CONS_SMEM_MAX;
     const size_t smem = lists ? with_lists : rid_label_cons_smem(S.N, C);
     const auto kern = lists ? k_label_cons<true> : k_label_cons<false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    static RidOnce once[2];
+    if (const cudaError_t e = rid_opt_in(once[lists], RID_SMEM_MOST, kern)) return e;
     ConsArgs A{S, R, C, B, n_steps, n_equil, step0, kT, x0, v0, pairs, d0, bsum, mf, se, sd, x_out, v_out, bad};
     kern<<<R, CT, smem, st>>>(A);
     return cudaGetLastError();

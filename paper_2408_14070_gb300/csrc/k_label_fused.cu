@@ -333,14 +333,8 @@ size_t rid_label_fused_smem(int N, int C, int threads) {
 
 template <int NT>
 static cudaError_t launch_nt(const FusedArgs& A, int grid, size_t smem, int P, cudaStream_t s) {
-    static unsigned long long attr = 0;
-    if (rid_first_on_device(attr)) {
-        cudaError_t e = cudaFuncSetAttribute(k_label_fused<NT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             220 * 1024);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_label_fused<NT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
-        if (e != cudaSuccess) return e;
-    }
+    static RidOnce once;
+    if (const cudaError_t e = rid_opt_in(once, 220 * 1024, k_label_fused<NT, false>, k_label_fused<NT, true>)) return e;
     if (P <= 1) {
         k_label_fused<NT, false><<<grid, NT, smem, s>>>(A, 1);
         return cudaGetLastError();

@@ -315,14 +315,11 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_label_run(FusedArgs A) {
 
 template <int NT>
 cudaError_t launch_run(const FusedArgs& A, int n_sm, size_t smem, cudaStream_t s) {
-    static unsigned long long attr = 0;
-    if (rid_first_on_device(attr)) {
-        const cudaError_t e =
-            cudaFuncSetAttribute(k_label_run<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, RUN_SMEM_MAX);
-        if (e != cudaSuccess) return e;
-    }
+    static RidOnce once;
+    cudaError_t e = rid_opt_in(once, RUN_SMEM_MAX, k_label_run<NT>);
+    if (e != cudaSuccess) return e;
     int occ = 0;
-    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_label_run<NT>, NT, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_label_run<NT>, NT, smem);
     if (e != cudaSuccess) return e;
     const long long most = (long long)(occ > 0 ? occ : 1) * n_sm;
     k_label_run<NT><<<(unsigned)(A.n_items < most ? A.n_items : most), NT, smem, s>>>(A);

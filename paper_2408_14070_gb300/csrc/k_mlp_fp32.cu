@@ -445,9 +445,9 @@ int choose_rpt(int wcn, int W, int M, int D, int H, int resnet, bool bwd) {
 
 template <int RPT, int WCN, bool BWD, bool SPLIT>
 void launch_f32(const MlpF32& E, int M, cudaStream_t s) {
-    static unsigned long long attr = 0;
+    static RidOnce once;
     auto k = k_mlp_fp32<RPT, WCN, BWD, SPLIT>;
-    if (rid_first_on_device(attr)) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, F32_SMEM_MAX);
+    rid_opt_in(once, F32_SMEM_MAX, k);
     constexpr int R = Shape<RPT, WCN>::R;
     k<<<dim3((E.W + R - 1) / R, M), NT, tile_smem(RPT, WCN, E.D, E.H, E.resnet, BWD), s>>>(E);
 }
@@ -666,11 +666,9 @@ void rid_launch_mlp_fp32(const EnsDev& E, StateDev st, int W, int C, cudaStream_
         while (sr < wpt) sr <<= 1;
         auto kern = sr == 1 ? k_mlp_fp32_small<1> : sr == 2 ? k_mlp_fp32_small<2> : sr == 4 ? k_mlp_fp32_small<4>
                   : sr == 8 ? k_mlp_fp32_small<8> : k_mlp_fp32_small<SR_MAX>;
-        static unsigned long long attr_small = 0;
-        if (rid_first_on_device(attr_small))
-            for (auto k : {k_mlp_fp32_small<1>, k_mlp_fp32_small<2>, k_mlp_fp32_small<4>, k_mlp_fp32_small<8>,
-                           k_mlp_fp32_small<SR_MAX>})
-                cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SM_MAX_FLOATS * 4);
+        static RidOnce once;
+        rid_opt_in(once, SM_MAX_FLOATS * 4, k_mlp_fp32_small<1>, k_mlp_fp32_small<2>, k_mlp_fp32_small<4>,
+                   k_mlp_fp32_small<8>, k_mlp_fp32_small<SR_MAX>);
         kern<<<dim3((W + tw - 1) / tw, E.M), NT, (size_t)Y.total * sizeof(float), s>>>(E, st, W, C, tw);
         return;
     }

@@ -450,17 +450,10 @@ cudaError_t rid_launch_mlp_tc(const TcArgs& P, const CUtensorMap& big, const CUt
     if (P.resnet && !P.rsave) return cudaErrorInvalidValue;
     const size_t smem = rid_mlp_tc_smem_bytes(P);
     const int v = (P.geb[0] == 1 ? 1 : 0) + (P.resnet ? 2 : 0);
-    static size_t attr[4][64] = {};   // shared memory opted into, per instantiation and device
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) dev = 0;
-    size_t& have = attr[v][dev & 63];
     auto kern = v == 0 ? k_mlp_tc<false, false> : v == 1 ? k_mlp_tc<true, false>
               : v == 2 ? k_mlp_tc<false, true> : k_mlp_tc<true, true>;
-    if (smem > have) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        have = smem;
-    }
+    static RidOnce once[4];
+    if (const cudaError_t e = rid_opt_in(once[v], RID_SMEM_MOST, kern)) return e;
     kern<<<dim3(P.ntiles, P.M, 1), NTHREADS, smem, s>>>(P, big, small);
     return cudaGetLastError();
 }

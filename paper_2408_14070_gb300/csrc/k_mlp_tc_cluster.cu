@@ -481,17 +481,10 @@ cudaError_t rid_launch_mlp_tc_cluster(const TcArgs& P, const CUtensorMap& big, c
     if (P.resnet && !P.rsave) return cudaErrorInvalidValue;
     const size_t smem = rid_mlp_tc_cluster_smem_bytes(P);
     const int v = (P.geb[0] == 1 ? 1 : 0) + (P.resnet ? 2 : 0);
-    static size_t attr[4][64] = {};   // shared memory opted into, per instantiation and device
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) dev = 0;
-    size_t& have = attr[v][dev & 63];
     auto kern = v == 0 ? k_mlp_tc_cluster<false, false> : v == 1 ? k_mlp_tc_cluster<true, false>
               : v == 2 ? k_mlp_tc_cluster<false, true> : k_mlp_tc_cluster<true, true>;
-    if (smem > have) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        have = smem;
-    }
+    static RidOnce once[4];
+    if (const cudaError_t e = rid_opt_in(once[v], RID_SMEM_MOST, kern)) return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(P.ntiles * P.csize, P.M, 1);
     cfg.blockDim = dim3(CL_THREADS, 1, 1);

@@ -647,17 +647,10 @@ cudaError_t launch_pair(TcArgs P, const CUtensorMap& big, const CUtensorMap& sma
     else if (smem < PAIR_SMEM_MIN) smem = PAIR_SMEM_MIN;
     if (ROWS == 128) P.ntiles = (P.ntiles + 1) / 2 * 2;   // the scratch buffers hold whole pairs of tiles
     const int v = (P.geb[0] == 1 ? 1 : 0) + (P.resnet ? 2 : 0);
-    static size_t attr[4][64] = {};   // shared memory opted into, per instantiation and device
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) dev = 0;
-    size_t& have = attr[v][dev & 63];
     auto kern = v == 0 ? k_mlp_tc_pair<false, false, ROWS> : v == 1 ? k_mlp_tc_pair<true, false, ROWS>
               : v == 2 ? k_mlp_tc_pair<false, true, ROWS> : k_mlp_tc_pair<true, true, ROWS>;
-    if (smem > have) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        have = smem;
-    }
+    static RidOnce once[4];
+    if (const cudaError_t e = rid_opt_in(once[v], PAIR_SMEM_MAX, kern)) return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(ROWS == 128 ? P.ntiles : 2 * P.ntiles, P.M, 1);
     cfg.blockDim = dim3(NTHREADS, 1, 1);

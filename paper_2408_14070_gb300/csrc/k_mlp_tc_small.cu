@@ -521,17 +521,10 @@ cudaError_t rid_launch_mlp_tc_small(const TcArgs& P, const CUtensorMap& big, con
         if (P.gN[g] > 128 * SM_MT) return cudaErrorInvalidValue;
     const size_t smem = rid_mlp_tc_small_smem_bytes(P, NW);
     const int v = (P.resnet ? 1 : 0) + (epi_warps == 8 ? 2 : 0);
-    static size_t attr[4][64] = {};   // shared memory opted into, per instantiation and device
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) dev = 0;
-    size_t& have = attr[v][dev & 63];
     auto kern = v == 0 ? k_mlp_tc_small<false, 16> : v == 1 ? k_mlp_tc_small<true, 16>
               : v == 2 ? k_mlp_tc_small<false, 8> : k_mlp_tc_small<true, 8>;
-    if (smem > have) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        have = smem;
-    }
+    static RidOnce once[4];
+    if (const cudaError_t e = rid_opt_in(once[v], RID_SMEM_MOST, kern)) return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(P.csize, P.M, 1);
     cfg.blockDim = dim3(sm_threads(epi_warps), 1, 1);

@@ -329,9 +329,11 @@ extern "C" RID_API int rid_select(const rid_select_desc* d, int32_t n, const flo
     k_sel_count<<<nb, SEL_T, 0, st>>>(deps, n, lo, hi, blk);
     k_sel_scan<<<1, SEL_T, 0, st>>>(blk, nb, dncand);
     k_sel_scatter<<<nb, SEL_T, 0, st>>>(dcv, deps, n, C, lo, hi, blk, cand, x, nn);
-    static unsigned long long attr = 0;
-    if (rid_first_on_device(attr))
-        cudaFuncSetAttribute(k_sel_leaders, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    static RidOnce once;
+    if ((e = rid_on_device(once, [](int) {
+             return cudaFuncSetAttribute(k_sel_leaders, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+         })) != cudaSuccess)
+        return sel_cuda(e, "cluster size");
     int hn[1 + SEL_TRIALS] = {};
     // nt clusterings side by side; their counts into hn[1 ..], the candidate count into hn[0]
     auto cluster = [&](const double* t, int nt, int stop, long long cap_l) -> int {

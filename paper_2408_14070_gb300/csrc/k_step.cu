@@ -462,10 +462,8 @@ void rid_launch_mb(const SysDev& S, StateDev st, int W, uint32_t step0, cudaStre
     if (n > 0) k_mb<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(S, st, W, step0);
 }
 void rid_launch_pair_mask(const SysDev& S, StateDev st, int W, uint32_t* mask, cudaStream_t s) {
-    static unsigned long long attr = 0;   // positions of up to RID_MAX_BEADS beads exceed the default 48 KB
-    if (rid_first_on_device(attr)) {
-        cudaFuncSetAttribute(k_pair_mask, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    }
+    static RidOnce once;   // positions of up to RID_MAX_BEADS beads exceed the default 48 KB
+    rid_opt_in(once, 200 * 1024, k_pair_mask);
     k_pair_mask<<<W, chain_threads(S.N), sizeof(float4) * (size_t)S.N, s>>>(S, st, mask);
 }
 
@@ -511,13 +509,8 @@ void rid_launch_ff(const SysDev& S, StateDev st, int W, bool energy, cudaStream_
     const int iters = (S.N + th - 1) / th;
     int ipc = iters;
     const int P = energy ? 1 : ff_split(W, iters, ipc);
-    static unsigned long long attr = 0;
-    if (rid_first_on_device(attr)) {
-        cudaFuncSetAttribute(k_ff<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        cudaFuncSetAttribute(k_ff<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        cudaFuncSetAttribute(k_ff<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        cudaFuncSetAttribute(k_ff<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    }
+    static RidOnce once;
+    rid_opt_in(once, 200 * 1024, k_ff<false, true>, k_ff<true, true>, k_ff<false, false>, k_ff<true, false>);
     const unsigned grid = (unsigned)W * (unsigned)P;
     if (bsm) {
         if (energy) k_ff<true, true><<<grid, th, sm, s>>>(S, st, P, ipc);
@@ -532,12 +525,9 @@ template <int MODE, bool FIN, bool KICK, int INT>
 static void head_e(const HeadArgs& a, cudaStream_t s) {
     const int th = HEAD_THREADS;
     const size_t sm = sizeof(float4) * (size_t)a.S.N + (FIN ? (sizeof(float4) + sizeof(int2)) * 4 * (size_t)a.S.C : 0);
-    static unsigned long long attr = 0;   // positions of up to RID_MAX_BEADS beads exceed the default 48 KB
-    if (rid_first_on_device(attr)) {
-        const int mx = (int)(sizeof(float4) * RID_MAX_BEADS + (sizeof(float4) + sizeof(int2)) * 4 * RID_MAX_CV);
-        cudaFuncSetAttribute(k_head<MODE, FIN, KICK, INT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-        cudaFuncSetAttribute(k_head<MODE, FIN, KICK, INT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-    }
+    static RidOnce once;   // positions of up to RID_MAX_BEADS beads exceed the default 48 KB
+    rid_opt_in(once, sizeof(float4) * RID_MAX_BEADS + (sizeof(float4) + sizeof(int2)) * 4 * RID_MAX_CV,
+               k_head<MODE, FIN, KICK, INT, true>, k_head<MODE, FIN, KICK, INT, false>);
     // CTAs per walker: a cluster over the bead batches with fewer walkers than two
     // per SM (not for energy launches, whose per-walker sums stay in one CTA, nor
     // for a server's jobs: under 16 concurrent jobs the clusters measured slower,

@@ -486,9 +486,8 @@ int tr_step(rid_trainer* tr, const int* idx, float* loss, int64_t step, const Ad
         u.eps = (float)d.adam_eps;
     }
     u.sums = (L + 1) * ((H + 255) / 256);
-    static unsigned long long attr = 0;
-    if (rid_first_on_device(attr))
-        cudaFuncSetAttribute(k_tr_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)UPD_SMEM);
+    static RidOnce once;
+    TCK(rid_opt_in(once, UPD_SMEM, k_tr_update));
     TCK(launch_k(k_tr_update, dim3(u.tile0[L] + u.sums + 1, M), dim3(256), UPD_SMEM, st, true, u));
     return RID_OK;
 }

@@ -409,17 +409,14 @@ __global__ void __launch_bounds__(TT) k_tr_big(GemmArgs g, EpiArgs e) {
 template <int EPI, bool KB>
 void launch_gemm(const GemmArgs& g, const EpiArgs& e, int M, cudaStream_t st, bool pdl) {
     if (g.rows >= 1024 && g.cols >= 64) {
-        static unsigned long long attr = 0;
-        if (rid_first_on_device(attr))
-            cudaFuncSetAttribute(k_tr_big<EPI, KB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BIG_SMEM);
+        static RidOnce once;
+        rid_opt_in(once, BIG_SMEM, k_tr_big<EPI, KB>);
         launch_k(k_tr_big<EPI, KB>, dim3((g.cols + BT - 1) / BT, (g.rows + BT - 1) / BT, M), dim3(TT), BIG_SMEM, st, pdl,
                  g, e);
         return;
     }
-    static unsigned long long attr = 0;
-    if (rid_first_on_device(attr))
-        cudaFuncSetAttribute(k_tr_tile<EPI, KB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(sizeof(float) * tile_floats(RID_MAX_WIDTH, KB)));
+    static RidOnce once;
+    rid_opt_in(once, sizeof(float) * tile_floats(RID_MAX_WIDTH, KB), k_tr_tile<EPI, KB>);
     launch_k(k_tr_tile<EPI, KB>, dim3((g.cols + 31) / 32, (g.rows + 31) / 32, M), dim3(TT),
              sizeof(float) * tile_floats(g.K, KB), st, pdl, g, e);
 }

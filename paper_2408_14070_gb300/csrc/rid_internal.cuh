@@ -7,6 +7,7 @@
 #include <stdint.h>
 
 #include "rid.h"
+#include "rid_once.cuh"
 
 // A named NVTX range over the lifetime of the object: each public call and
 // each server tick shows as one range in a profiler that records NVTX (a
@@ -199,16 +200,39 @@ __device__ __forceinline__ double rid_cv_offset(int4 q, double s, double s0) {
 }
 
 // --------------------------------------------------------------------------
-// cudaFuncSetAttribute acts on the current device only: a launcher that opts
-// a kernel into more shared memory asks this first, and it answers true once
-// per device (one bit of `done` per device ordinal).
-inline bool rid_first_on_device(unsigned long long& done) {
+// Set-up of kernels on the current device, once per device for all threads.
+template <typename F>
+cudaError_t rid_on_device(RidOnce& once, F set) {
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return true;
-    const unsigned long long bit = 1ull << (dev & 63);
-    if (done & bit) return false;
-    done |= bit;
-    return true;
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    return (cudaError_t)rid_once(once, dev, [&] { return (int)set(dev); });
+}
+// The shared memory that a kernel is opted into belongs to the process, so a
+// launcher opts in once, for the most that any of its launches asks for: a
+// smaller size set by one thread would fail another thread's launch.  `bytes`
+// of dynamic shared memory; 0: all that the device gives beside the kernel's
+// static arrays.
+constexpr size_t RID_SMEM_MOST = 0;
+template <typename K>
+cudaError_t rid_smem_attr(int dev, size_t bytes, K kernel) {
+    if (bytes == RID_SMEM_MOST) {
+        int most = 0;
+        cudaFuncAttributes fa{};
+        cudaError_t e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kernel);
+        if (e != cudaSuccess) return e;
+        bytes = (size_t)most - fa.sharedSizeBytes;
+    }
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+template <typename... K>
+cudaError_t rid_opt_in(RidOnce& once, size_t bytes, K... kernels) {
+    return rid_on_device(once, [&](int dev) {
+        cudaError_t e = cudaSuccess;
+        ((e = e == cudaSuccess ? rid_smem_attr(dev, bytes, kernels) : e), ...);
+        return e;
+    });
 }
 
 // --------------------------------------------------------------------------
