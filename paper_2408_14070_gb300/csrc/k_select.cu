@@ -88,11 +88,15 @@ __global__ void __launch_bounds__(SEL_T) k_sel_count(const float* __restrict__ e
     if (threadIdx.x == 0) blk[blockIdx.x] = c;
 }
 
-// Exclusive prefix sums of blk[nb] in place; the total into *n_cand.
-__global__ void __launch_bounds__(SEL_T) k_sel_scan(int* __restrict__ blk, int nb, int* __restrict__ n_cand) {
+// Exclusive prefix sums of blk[nb] in place; the total into *n_cand.  Clears
+// the word that the trials of each later launch share.
+constexpr int SEL_LAUNCHES = 66;   // 64 trials at most, then the clustering kept
+__global__ void __launch_bounds__(SEL_T) k_sel_scan(int* __restrict__ blk, int nb, int* __restrict__ n_cand,
+                                                    unsigned* __restrict__ out_words) {
     __shared__ int warp_sums[32];
     __shared__ int tot;
     int base = 0;
+    if (threadIdx.x < SEL_LAUNCHES) out_words[threadIdx.x] = 0;
     for (int b0 = 0; b0 < nb; b0 += SEL_T) {
         const int b = b0 + threadIdx.x;
         const int v = b < nb ? blk[b] : 0;
@@ -141,12 +145,15 @@ __device__ __forceinline__ void sel_cluster_sync() {
 }
 
 // The trials of one launch: thresholds (squared, FP32), where a trial stops
-// (0: runs to the end), and its leader list at lead + trial * lcap.
+// (0: runs to the end), its leader list at lead + trial * lcap, and the trials
+// (bits) that the search no longer visits once this one has found more than
+// `upper` clusters, fewer than `lower`, or a count between them.
 constexpr int SEL_TRIALS = 7;
 constexpr int SEL_CLUSTER = 16;
 struct SelTrials {
     float t2[SEL_TRIALS];
-    int stop;
+    int stop, lower, upper;
+    unsigned many_out[SEL_TRIALS], few_out[SEL_TRIALS], hit_out[SEL_TRIALS];
 };
 
 // One trial per cluster of P CTAs (CTAs trial * P ..).  Candidate k belongs to
@@ -161,15 +168,22 @@ struct SelTrials {
 // A round is bound by latency (the leader's CVs from L2, two block barriers and
 // a cluster barrier), its distances being spread over 16 SMs.  102400 frames x
 // 20 CVs searched into 30-45 clusters: 14.9 ms a call with one CTA settling
-// 1024 candidates at a time and the trials one after another, 0.83 ms now.
+// 1024 candidates at a time and the trials one after another, 0.71 ms now.
+// A trial that ends sets the bits of those it makes needless in *out, and these
+// leave: the first CTA of a cluster reads the word every eighth round, uses it
+// four rounds later (a read takes longer than a short round) and sends 0 in its
+// next message, so that the cluster leaves together.  (Without it a
+// search whose first trial is already in a wide window, 10 clusters in 1 to
+// 20000, waited for trials that count to 20001: 48.9 ms at 102400 frames of 20
+// CVs, 2.6 ms now, 25.8 ms with one trial at a time in one CTA.)
 // Candidates past the first 32 of a thread keep their bits in alive_g
 // [trial][word - 1][1024 P].
 __global__ void __launch_bounds__(SEL_T) k_sel_leaders(const float* __restrict__ x, long long cap,
                                                        const int* __restrict__ n_cand_p, int C,
                                                        const float* __restrict__ w, const int* __restrict__ per,
                                                        SelTrials T, int P, int* __restrict__ lead, long long lcap,
-                                                       int* __restrict__ n_lead, unsigned* __restrict__ alive_g,
-                                                       long long alive_stride) {
+                                                       int* __restrict__ n_lead, unsigned* out,
+                                                       unsigned* __restrict__ alive_g, long long alive_stride) {
     __shared__ float lc[RID_MAX_CV], ws[RID_MAX_CV];
     __shared__ int ps[RID_MAX_CV];
     __shared__ unsigned wmin[32];
@@ -192,7 +206,8 @@ __global__ void __launch_bounds__(SEL_T) k_sel_leaders(const float* __restrict__
     };
     unsigned word0 = full_word(0);
     for (unsigned q = 1; q < words; ++q) alive[(long long)(q - 1) * G] = full_word(q);
-    unsigned first = mine ? g : NONE;
+    unsigned first = mine ? g + 1 : NONE;                       // 1 + this thread's smallest candidate left
+    unsigned gone = 0, seen = 0;                                // *out, in the cluster's first thread
     int nl = 0, par = 0;
     // every CTA of the cluster runs before a peer writes to its shared memory
     if (P > 1) sel_cluster_sync();
@@ -201,7 +216,8 @@ __global__ void __launch_bounds__(SEL_T) k_sel_leaders(const float* __restrict__
         if (lane == 0) wmin[warp] = v;
         __syncthreads();
         if (warp == 0) {
-            v = __reduce_min_sync(0xffffffffu, wmin[lane]);
+            // the message: 1 + the candidate, NONE, or 0 to leave
+            v = __reduce_min_sync(0xffffffffu, gone >> trial & 1u ? 0u : wmin[lane]);
             if (P == 1) {
                 if (lane == 0) cmin[par][0] = v;
             } else if (lane < P) {
@@ -215,11 +231,17 @@ __global__ void __launch_bounds__(SEL_T) k_sel_leaders(const float* __restrict__
         for (int q = 0; q < P; ++q) L = min(L, cmin[par][q]);
         par ^= 1;                     // this parity is written again only after the next barrier
         if (L == NONE) break;
+        if (L == 0) return;           // the same in every thread of the cluster, after its barrier
+        --L;
         if (rank == 0 && tid == 0 && nl < lcap) lead[trial * lcap + nl] = (int)L;
         ++nl;
         if (T.stop > 0 && nl > T.stop) break;
         if (tid < C) lc[tid] = x[tid * cap + L];
         __syncthreads();
+        if (rank == 0 && tid == 0) {
+            if (nl % 8 == 0) seen = *reinterpret_cast<const volatile unsigned*>(out);
+            else if (nl % 8 == 4) gone = seen;
+        }
         first = NONE;
         for (unsigned q = 0; q < words; ++q) {
             unsigned a = q == 0 ? word0 : alive[(long long)(q - 1) * G];
@@ -230,12 +252,16 @@ __global__ void __launch_bounds__(SEL_T) k_sel_leaders(const float* __restrict__
                 const unsigned k = g + G * (32 * q + b);
                 if (k == L || sel_d2(lc, x + k, cap, ws, ps, C) <= t2) a &= ~(1u << b);
             }
-            if (a && first == NONE) first = g + G * (32 * q + __ffs(a) - 1);
+            if (a && first == NONE) first = g + G * (32 * q + __ffs(a) - 1) + 1;
             if (q == 0) word0 = a;
             else if (a != was) alive[(long long)(q - 1) * G] = a;
         }
     }
-    if (rank == 0 && tid == 0) n_lead[trial] = nl;
+    if (rank == 0 && tid == 0) {
+        n_lead[trial] = nl;
+        const unsigned rest = nl > T.upper ? T.many_out[trial] : nl < T.lower ? T.few_out[trial] : T.hit_out[trial];
+        if (rest) atomicOr(out, rest);
+    }
 }
 
 // selected[i] = frame index of leader i (leaders hold candidate rows)
@@ -291,7 +317,7 @@ extern "C" RID_API int rid_select(const rid_select_desc* d, int32_t n, const flo
     const long long awords = ((nn + G - 1) / G + 31) / 32 - 1;
     const long long ncv = mem == RID_MEM_HOST ? nn * C : 0, neps = mem == RID_MEM_HOST ? nn : 0;
     const size_t bytes = sizeof(float) * (size_t)(ncv + neps + nn * C + C) +
-                         sizeof(int) * (size_t)(nn + nlead + nb + C + 1 + trials + trials * awords * G + nn);
+                         sizeof(int) * (size_t)(nn + nlead + nb + C + 1 + trials + SEL_LAUNCHES + trials * awords * G + nn);
     SelBuf buf;
     if (cudaMalloc(&buf.p, bytes) != cudaSuccess) {
         cudaGetLastError();
@@ -307,7 +333,8 @@ extern "C" RID_API int rid_select(const rid_select_desc* d, int32_t n, const flo
     int* dper = blk + nb;
     int* dncand = dper + C;                          // then the leader counts of a launch's trials
     int* dnl = dncand + 1;
-    unsigned* alive = reinterpret_cast<unsigned*>(dnl + trials);
+    unsigned* out_words = reinterpret_cast<unsigned*>(dnl + trials);   // one per launch
+    unsigned* alive = out_words + SEL_LAUNCHES;
     int* dsel_buf = reinterpret_cast<int*>(alive + trials * awords * G);   // [nn] frame indices of the selection
     cudaError_t e;
     const float* dcv = cv;
@@ -327,7 +354,7 @@ extern "C" RID_API int rid_select(const rid_select_desc* d, int32_t n, const flo
     // trust window: eps in [lo, hi), compared in FP32 (the eps values are FP32)
     const float lo = (float)d->trust_lo, hi = (float)d->trust_hi;
     k_sel_count<<<nb, SEL_T, 0, st>>>(deps, n, lo, hi, blk);
-    k_sel_scan<<<1, SEL_T, 0, st>>>(blk, nb, dncand);
+    k_sel_scan<<<1, SEL_T, 0, st>>>(blk, nb, dncand, out_words);
     k_sel_scatter<<<nb, SEL_T, 0, st>>>(dcv, deps, n, C, lo, hi, blk, cand, x, nn);
     static RidOnce once;
     if ((e = rid_on_device(once, [](int) {
@@ -336,8 +363,8 @@ extern "C" RID_API int rid_select(const rid_select_desc* d, int32_t n, const flo
         return sel_cuda(e, "cluster size");
     int hn[1 + SEL_TRIALS] = {};
     // nt clusterings side by side; their counts into hn[1 ..], the candidate count into hn[0]
-    auto cluster = [&](const double* t, int nt, int stop, long long cap_l) -> int {
-        SelTrials T{};
+    int n_launch = 0;
+    auto cluster = [&](SelTrials T, const double* t, int nt, int stop, long long cap_l) -> int {
         for (int k = 0; k < nt; ++k) T.t2[k] = (float)(t[k] * t[k]);
         T.stop = stop;
         cudaLaunchConfig_t cfg{};
@@ -352,8 +379,8 @@ extern "C" RID_API int rid_select(const rid_select_desc* d, int32_t n, const flo
         cfg.attrs = at;
         cfg.numAttrs = 1;
         cudaError_t e2 = cudaLaunchKernelEx(&cfg, k_sel_leaders, (const float*)x, nn, (const int*)dncand, C,
-                                            (const float*)dw, (const int*)dper, T, P, lead, cap_l, dnl, alive,
-                                            awords * G);
+                                            (const float*)dw, (const int*)dper, T, P, lead, cap_l, dnl,
+                                            out_words + n_launch++, alive, awords * G);
         if (e2 != cudaSuccess) return sel_cuda(e2, "launch");
         if ((e2 = cudaMemcpyAsync(hn, dncand, sizeof(int) * (1 + nt), cudaMemcpyDeviceToHost, st)) != cudaSuccess)
             return sel_cuda(e2, "count");
@@ -364,7 +391,7 @@ extern "C" RID_API int rid_select(const rid_select_desc* d, int32_t n, const flo
     int count = 0;
     const int* leaders = lead;
     if (!d->adapt) {
-        if (int rc = cluster(&t, 1, 0, lcap)) return rc;
+        if (int rc = cluster({}, &t, 1, 0, lcap)) return rc;
         count = hn[1];
     } else {
         // The search: t doubles or halves until the count is bracketed, then
@@ -404,8 +431,18 @@ extern "C" RID_API int rid_select(const rid_select_desc* d, int32_t n, const flo
                         (many ? tree[k].many : tree[k].few) = nt;
                         tree[nt++] = step(tree[k], many != 0);
                     }
-            for (int k = 0; k < nt; ++k) tt[k] = tree[k].t;
-            if (int rc = cluster(tt, nt, upper, lcap)) return rc;
+            SelTrials T{};
+            T.lower = lower;
+            T.upper = upper;
+            unsigned below[SEL_TRIALS];          // a node and all after it (children follow their parents)
+            for (int k = nt - 1; k >= 0; --k) {
+                T.few_out[k] = tree[k].many < 0 ? 0u : below[tree[k].many];
+                T.many_out[k] = tree[k].few < 0 ? 0u : below[tree[k].few];
+                T.hit_out[k] = T.few_out[k] | T.many_out[k];
+                below[k] = 1u << k | T.hit_out[k];
+                tt[k] = tree[k].t;
+            }
+            if (int rc = cluster(T, tt, nt, upper, lcap)) return rc;
             for (at = 0;;) {
                 t = tree[at].t;
                 count = hn[1 + at];
@@ -425,7 +462,7 @@ extern "C" RID_API int rid_select(const rid_select_desc* d, int32_t n, const flo
         }
         leaders = lead + at * lcap;
         if (count > upper) {   // the clustering finally kept had stopped early
-            if (int rc = cluster(&t, 1, 0, nn)) return rc;
+            if (int rc = cluster({}, &t, 1, 0, nn)) return rc;
             count = hn[1];
             leaders = lead;
         }

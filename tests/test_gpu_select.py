@@ -98,3 +98,46 @@ def test_cluster_ownership_edges(R, n, C, thr, lower, upper, adapt):
     ref = S.select(cv, eps, 0.0, 5.0, thr, lower, upper, adapt, 64)
     assert (nc, t) == (ref["n_clusters"], ref["threshold"])
     np.testing.assert_array_equal(sel, ref["selected"])
+
+
+def test_wide_window_ends_with_its_first_trial(R):
+    # A search whose first trial lies in the window needs that clustering alone: a few clusters here, in a
+    # window to 10000 that the smaller thresholds tried ahead would take hundreds of rounds over.  Four times the
+    # time of the same clustering without a search leaves room for the launches' ends.
+    import time
+    import torch
+    n, C = 60000, 6
+    cv, eps = _frames(n, C, 9, walkers=1)
+    dc, de = torch.from_numpy(cv).cuda(), torch.from_numpy(eps).cuda()
+    out = torch.zeros(64, dtype=torch.int32, device="cuda")
+    thr = 4.0
+
+    def best(lower, upper, adapt):
+        t = []
+        for _ in range(6):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            res = R.select(dc, de, 0.0, 5.0, thr, lower, upper, adapt, 64, selected=out)
+            t.append(time.perf_counter() - t0)
+        return min(t), res
+
+    plain, (_, n_plain, _) = best(1, 1 << 30, False)
+    wide, (_, n_wide, t_wide) = best(1, 10000, True)
+    assert 2 <= n_plain <= 200 and (n_wide, t_wide) == (n_plain, thr)
+    assert wide < 4 * plain, (wide, plain)
+
+
+@pytest.mark.parametrize("n,lower,upper,thr", [
+    (3000, 1, 2000, 2.0),       # one CTA a trial, the first trial in a wide window
+    (10000, 900, 1000, 4.0),    # clusters; too few at first, then trials that run for long
+    (10000, 4, 6, 0.4),         # too many at first
+    (10000, 1, 1 << 30, 0.05),  # a window that nothing leaves
+])
+def test_trials_that_leave_early_change_nothing(R, n, lower, upper, thr):
+    # (equality with the oracle, as above: no tolerance)
+    cv, eps = _frames(n, 3, n + lower, walkers=1)
+    for _ in range(3):
+        sel, nc, t = R.select(cv, eps, 0.0, 5.0, thr, lower, upper, True, 64)
+    ref = S.select(cv, eps, 0.0, 5.0, thr, lower, upper, True, 64)
+    assert (nc, t) == (ref["n_clusters"], ref["threshold"])
+    np.testing.assert_array_equal(sel, ref["selected"])
