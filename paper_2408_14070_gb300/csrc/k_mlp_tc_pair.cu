@@ -19,8 +19,7 @@
 // instruction, the saved tanh two steps ahead, keeps the residual stream in
 // TMEM where two accumulators fit, and saves a plain BF16 layer's tanh from the
 // operand tile after releasing it, while the MMAs run.  The release to the
-// even CTA is an arrive without cluster-scope ordering: with it every GEMM
-// waited for the saved activations to reach L2 (4 us of 47 a launch).
+// even CTA orders shared memory alone (pair_arrive).
 // Measured per launch, one CTA per 128 walkers before -> pairs of 128 rows:
 // 8 x 64-512x4-1 at 8192 walkers 436 -> 315 us (682 of 1873 TFLOP/s), 4 x
 // 40-256x4-1 at 8192 walkers 79 -> 73 us, residual 127 -> 94 us; pairs of 64 rows,
@@ -79,11 +78,26 @@ __device__ __forceinline__ void pair_tma_load(uint32_t dst, const CUtensorMap* m
         "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(row), "r"(leader_bar)
         : "memory");
 }
-// Arrive on a barrier of the even CTA.  What it orders is this CTA's shared memory, which fence.proxy.async
-// before it has already handed to the MMAs: a release at cluster scope would also wait for the saved
-// activations' way to L2.
+// Hand this CTA's rows of an operand to the even CTA, whose MMAs read them: release at cluster scope of
+// shared memory alone, before a relaxed arrive (the writers have handed it to the async proxy already).  An
+// arrive that releases all memory costs half a microsecond a GEMM here, also from a thread that has written
+// nothing: 30.5 -> 34.2 us a launch (128 walkers of 4 x 40-256x4-1), 30.6 with this fence.
 __device__ __forceinline__ void pair_arrive(uint32_t local_bar) {
-    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(mapa(local_bar, 0)) : "memory");
+    asm volatile("fence.release.sync_restrict::shared::cta.cluster;" ::: "memory");
+    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(mapa(local_bar, 0)) : "memory");
+}
+// The even CTA's wait for it: relaxed, then an acquire of shared memory alone.
+__device__ __forceinline__ bool pair_try(uint32_t a, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{ .reg .pred p; mbarrier.try_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+        : "=r"(ok)
+        : "r"(a), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ void pair_acquire() {
+    asm volatile("fence.acquire.sync_restrict::shared::cluster.cluster;" ::: "memory");
 }
 // Sixteen 32-bit columns of this thread's TMEM lane, from or to registers.
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
@@ -369,10 +383,11 @@ __global__ void __maxnreg__(96)
                 const bool f8 = F8 && P.geb[g] == 1;
                 // completion g of a_full: both CTAs' input for g = 0, then their epilogues of GEMM
                 // g - 1, which have also read the accumulator
-                if (!mbar_wait(smem_u32(&S.a_full), g & 1, abort_flag, P.err, 4)) {
+                if (!mbar_wait_by<pair_try>(smem_u32(&S.a_full), g & 1, abort_flag, P.err, 4)) {
                     ok = false;
                     break;
                 }
+                pair_acquire();
                 fence_after();
                 for (int n0 = 0; n0 < N && ok; n0 += 256) {
                     const int rows = N - n0 < 256 ? N - n0 : 256;

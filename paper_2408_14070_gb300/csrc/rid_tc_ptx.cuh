@@ -45,11 +45,12 @@ __device__ __forceinline__ bool mbar_try(uint32_t a, uint32_t parity) {
     return ok != 0;
 }
 // Bounded wait: false if the deadline passed or another role aborted.
-__device__ __forceinline__ bool mbar_wait(uint32_t a, uint32_t parity, volatile int* abort_flag, int* err, int code) {
-    if (mbar_try(a, parity)) return true;
+template <bool (*TRY)(uint32_t, uint32_t)>
+__device__ __forceinline__ bool mbar_wait_by(uint32_t a, uint32_t parity, volatile int* abort_flag, int* err, int code) {
+    if (TRY(a, parity)) return true;
     const unsigned long long t0 = gtimer();
     while (true) {
-        if (mbar_try(a, parity)) return true;
+        if (TRY(a, parity)) return true;
         if (*abort_flag) return false;
         if (gtimer() - t0 > WAIT_NS) {
             *abort_flag = 1;
@@ -57,6 +58,9 @@ __device__ __forceinline__ bool mbar_wait(uint32_t a, uint32_t parity, volatile 
             return false;
         }
     }
+}
+__device__ __forceinline__ bool mbar_wait(uint32_t a, uint32_t parity, volatile int* abort_flag, int* err, int code) {
+    return mbar_wait_by<mbar_try>(a, parity, abort_flag, err, code);
 }
 
 // tcgen05 shared-memory matrix descriptor for a K-major operand in the
@@ -235,17 +239,7 @@ __device__ __forceinline__ bool mbar_try_cluster(uint32_t a, uint32_t parity) {
 // Bounded wait on a barrier that other CTAs of the cluster arrive on.
 __device__ __forceinline__ bool mbar_wait_cluster(uint32_t a, uint32_t parity, volatile int* abort_flag, int* err,
                                                   int code) {
-    if (mbar_try_cluster(a, parity)) return true;
-    const unsigned long long t0 = gtimer();
-    while (true) {
-        if (mbar_try_cluster(a, parity)) return true;
-        if (*abort_flag) return false;
-        if (gtimer() - t0 > WAIT_NS) {
-            *abort_flag = 1;
-            atomicOr(err, code);
-            return false;
-        }
-    }
+    return mbar_wait_by<mbar_try_cluster>(a, parity, abort_flag, err, code);
 }
 __device__ __forceinline__ void fence_async_smem_cluster() {
     asm volatile("fence.proxy.async.shared::cluster;" ::: "memory");
