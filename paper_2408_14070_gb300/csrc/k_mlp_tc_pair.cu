@@ -28,6 +28,7 @@
 // the epilogue, 38 without both and the weights: hand-overs, saves and the call's
 // ends.  Measured and not kept: the second 256 columns' MMAs under the first's
 // epilogue, its results parked in TMEM (319 -> 310 us, and 5% slower to 256 columns).
+#include "rid_pair_loads.cuh"
 #include "rid_tc_ptx.cuh"
 
 namespace {
@@ -40,6 +41,9 @@ struct Smem {
     uint64_t drain;
     uint32_t tmem_base;
     int abort_flag;
+    int issued;                      // weight iterations whose part this CTA has issued
+    int odd_issued;                  // even CTA: the odd CTA's, and in both CTAs the other one's abort flag
+    int peer_abort;
 };
 
 constexpr uint32_t PAIR_STAGE = 128u * 128u;   // half of a 256-row weight chunk
@@ -238,6 +242,45 @@ __device__ __forceinline__ float pair_member_value(const TcArgs& P, int m, int t
     return a + __ldg(P.bout + m);
 }
 
+// Rows of the weight chunk of iteration `it`, and the even CTA's share of them.
+template <bool F8>
+__device__ __noinline__ void chunk_rows(const TcArgs& P, int it, int& rows, int& half) {
+    rows = half = 0;
+    for (int g = 0; g < P.ngemm; ++g) {
+        const int N = P.gN[g], nch = P.gKp[g] * (F8 ? P.geb[g] : 2) / 128;
+        for (int n0 = 0; n0 < N; n0 += 256, it -= nch)
+            if (it < nch) {
+                rows = N - n0 < 256 ? N - n0 : 256;
+                half = min((rows + 31) / 32 * 16, rows);
+                return;
+            }
+    }
+}
+// After a wait has run out (one thread of the even CTA, both CTAs past their
+// roles): until the loads that either CTA has issued have landed, or the limit.
+// A part that was not issued is counted as if it had landed, so that the
+// stage's phase ends with the part that was.
+template <bool F8>
+__device__ __noinline__ void land_loads(const TcArgs& P, Smem& S) {
+    const unsigned long long t0 = gtimer();
+    for (int s = 0; s < P.stages; ++s) {
+        const PairStageLoads q = pair_stage_loads(S.issued, S.odd_issued, P.stages, s);
+        if (q.it < 0) continue;
+        const uint32_t bar = smem_u32(&S.full[s]);
+        if (q.even != q.odd) {
+            int rows, half;
+            chunk_rows<F8>(P, q.it, rows, half);
+            if (q.even)
+                asm volatile("mbarrier.complete_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar),
+                             "r"((uint32_t)(rows - half) * 128u)
+                             : "memory");
+            else
+                mbar_arrive_tx(bar, (uint32_t)(rows - half) * 128u);
+        }
+        while (!mbar_try(bar, (q.it / P.stages) & 1) && gtimer() - t0 < 2 * WAIT_NS) {}
+    }
+}
+
 // 18 warps spread 5/5/4/4 over the four schedulers, each with 16K registers:
 // at most 96 registers per thread
 // F8: the forward GEMMs take FP8 e4m3 operands (the input-gradient GEMMs
@@ -276,6 +319,9 @@ __global__ void __maxnreg__(96)
         mbar_init(smem_u32(&S.a_full), 2 * EPI_WARPS);
         mbar_init(smem_u32(&S.drain), 1);
         S.abort_flag = 0;
+        S.issued = 0;
+        S.odd_issued = 0;
+        S.peer_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncwarp();
@@ -333,8 +379,6 @@ __global__ void __maxnreg__(96)
         // ------------------------------------------------------------ TMA producer
         if (lane == 0) {
             int it = 0;
-            int last_it[TC_MAX_STAGES];
-            for (int s = 0; s < NS; ++s) last_it[s] = -1;
             bool ok = true;
             // (N is a multiple of 32: both CTAs load part of every stage, so neither runs ahead of the other)
             for (int g = 0; g < G && ok; ++g) {
@@ -349,10 +393,7 @@ __global__ void __maxnreg__(96)
                             ok = false;
                             break;
                         }
-                        if (rank == 0) {
-                            mbar_arrive_tx(smem_u32(&S.full[s]), (uint32_t)rows * 128u);
-                            last_it[s] = it;
-                        }
+                        if (rank == 0) mbar_arrive_tx(smem_u32(&S.full[s]), (uint32_t)rows * 128u);
                         const uint32_t bar = mapa(smem_u32(&S.full[s]), 0);
                         const long long first =
                             (long long)m * P.member_rows + P.grow[g] + (long long)c * N + n0 + (rank == 0 ? 0 : half);
@@ -364,14 +405,7 @@ __global__ void __maxnreg__(96)
                     }
                 }
             }
-            if (!ok) {
-                // the loads already issued land before a CTA of the pair can exit
-                for (int s = 0; s < NS; ++s)
-                    if (last_it[s] >= 0) {
-                        const unsigned long long t0 = gtimer();
-                        while (!mbar_try(smem_u32(&S.full[s]), (last_it[s] / NS) & 1) && gtimer() - t0 < WAIT_NS) {}
-                    }
-            }
+            S.issued = it;
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer (even CTA)
@@ -634,8 +668,18 @@ __global__ void __maxnreg__(96)
         if ((ROWS == 128 || hf == 0) && valid && !S.abort_flag)
             P.Apart[(size_t)m * P.W + wg] = pair_member_value(P, m, tile, row);
     }
+    if (threadIdx.x == 0 && S.abort_flag) {
+        const uint32_t other = rank ^ 1u;
+        st_cluster_u32(mapa(smem_u32(&S.peer_abort), other), 1u);
+    }
+    if (threadIdx.x == 0 && rank == 1) st_cluster_u32(mapa(smem_u32(&S.odd_issued), 0), (uint32_t)S.issued);
     __syncwarp();
-    cluster_sync_all();               // no CTA leaves while the pair's MMAs or loads may touch it
+    cluster_sync_all();               // no CTA leaves while the pair's MMAs may touch it
+    if (S.abort_flag || S.peer_abort) {   // the same in both CTAs
+        if (rank == 0 && threadIdx.x == 0) land_loads<F8>(P, S);
+        __syncwarp();
+        cluster_sync_all();           // ... nor while loads that no MMA has waited for are on their way
+    }
     if (warp == 1) {
         fence_after();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)P.tmem_cols)

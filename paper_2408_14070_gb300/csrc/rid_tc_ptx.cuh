@@ -219,6 +219,9 @@ __device__ __forceinline__ void st_cluster_v4(uint32_t a, uint4 v) {
 __device__ __forceinline__ void st_cluster_v2(uint32_t a, uint2 v) {
     asm volatile("st.shared::cluster.v2.b32 [%0], {%1, %2};" ::"r"(a), "r"(v.x), "r"(v.y) : "memory");
 }
+__device__ __forceinline__ void st_cluster_u32(uint32_t a, uint32_t v) {
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
 __device__ __forceinline__ void st_cluster_f32(uint32_t a, float v) {
     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
 }
