@@ -301,7 +301,9 @@ __global__ void __maxnreg__(96)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_rank();
     const int m = blockIdx.y;
-    // the 128-row tile of the scratch buffers that holds this CTA's rows, and their first row in it
+    // the 128-row tile of the scratch buffers that holds this CTA's rows, and their first row in it.  (With an
+    // odd number of tiles the last pair's second CTA has none: it streams its half of the weights, its rows are
+    // zeros that nothing reads, and its epilogue has no columns.)
     const int tile = ROWS == 128 ? blockIdx.x : blockIdx.x >> 1;
     const int row0 = ROWS == 128 ? 0 : (int)rank * 64;
     const int L = P.L, G = P.ngemm;   // 2L, or L for the member values alone
@@ -499,7 +501,7 @@ __global__ void __maxnreg__(96)
                 ng0 = max(ng0, 0);
                 ng1 = max(ng1, 0);
             }
-            const int ngr = ng0 + ng1, gpw = (ngr + 3) / 4;
+            const int ngr = tile < P.ntiles ? ng0 + ng1 : 0, gpw = (ngr + 3) / 4;
             const int i0 = min(sub * gpw, ngr), i1 = min(i0 + gpw, ngr);
             auto col_of = [&](int i) {
                 if (ROWS == 128) return 16 * i;
@@ -704,14 +706,13 @@ cudaError_t launch_pair(TcArgs P, const CUtensorMap& big, const CUtensorMap& sma
     while (P.tmem_cols < cols) P.tmem_cols *= 2;
     if (P.tmem_cols > 256) smem = PAIR_SMEM_MAX;
     else if (smem < PAIR_SMEM_MIN) smem = PAIR_SMEM_MIN;
-    if (ROWS == 128) P.ntiles = (P.ntiles + 1) / 2 * 2;   // the scratch buffers hold whole pairs of tiles
     const int v = (P.geb[0] == 1 ? 1 : 0) + (P.resnet ? 2 : 0);
     auto kern = v == 0 ? k_mlp_tc_pair<false, false, ROWS> : v == 1 ? k_mlp_tc_pair<true, false, ROWS>
               : v == 2 ? k_mlp_tc_pair<false, true, ROWS> : k_mlp_tc_pair<true, true, ROWS>;
     static RidOnce once[4];
     if (const cudaError_t e = rid_opt_in(once[v], PAIR_SMEM_MAX, kern)) return e;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(ROWS == 128 ? P.ntiles : 2 * P.ntiles, P.M, 1);
+    cfg.gridDim = dim3(ROWS == 128 ? (P.ntiles + 1) / 2 * 2 : 2 * P.ntiles, P.M, 1);
     cfg.blockDim = dim3(NTHREADS, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;

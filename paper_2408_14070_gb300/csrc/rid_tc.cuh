@@ -11,8 +11,8 @@
 #define TC_MAX_KCHUNKS 8   // 128-byte K-chunks of the widest GEMM (K <= 512 BF16)
 #define TC_MAX_QSLICES 32  // 16-column slices of the widest hidden layer (512)
 
-// Tiles of 128 walkers in the scratch buffers: whole pairs of them, for the kernel whose CTAs come in pairs.
-inline size_t rid_tc_tiles(int W) { return ((size_t)W + 255) / 256 * 2; }
+// Tiles of 128 walkers in the scratch buffers.
+inline size_t rid_tc_tiles(int W) { return ((size_t)W + 127) / 128; }
 
 // Weight image, per member: for GEMM g (forward layers 0..L-1, then backward
 // layers L-1..0) and K-chunk c (128 bytes of K: 64 BF16 or 128 FP8 e4m3
