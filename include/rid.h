@@ -597,7 +597,7 @@ typedef struct {
  * all of its steps.  Jobs may differ in chain length, CV count, restraints and step counts.
  * Each job's outputs are bit-identical to rid_label on the same inputs.
  *   threads     CTA size of every run: 128, 256 or 512, or 0 to choose it by
- *               chain length
+ *               chain length, shared memory and number of runs
  *   status_out  [n_jobs] | NULL: per job RID_OK or RID_ERR_NONFINITE
  * `mem` applies to every array of every job.  Synchronous.  The jobs' device
  * memory comes from the server pool and is released before the call returns.

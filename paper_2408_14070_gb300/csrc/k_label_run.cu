@@ -22,6 +22,8 @@
 // k_label_fused, 0.58 now; 512 uneven runs of 50 to 500 beads x 250 steps, the
 // call in C: 6.4 ms and 4.6 (k_label_fused's CTA size chosen by timing, the
 // longest chain's shared memory for all).
+#include <cmath>
+
 #include "rid_batch.cuh"
 #include "rid_forces.cuh"
 
@@ -313,14 +315,19 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_label_run(FusedArgs A) {
     }
 }
 
+// Runs that an SM holds at once.
 template <int NT>
-cudaError_t launch_run(const FusedArgs& A, int n_sm, size_t smem, cudaStream_t s) {
+cudaError_t runs_per_sm(size_t smem, int& occ) {
     static RidOnce once;
     cudaError_t e = rid_opt_in(once, RUN_SMEM_MAX, k_label_run<NT>);
-    if (e != cudaSuccess) return e;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_label_run<NT>, NT, smem);
+    return e;
+}
+
+template <int NT>
+cudaError_t launch_run(const FusedArgs& A, int n_sm, size_t smem, cudaStream_t s) {
     int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_label_run<NT>, NT, smem);
-    if (e != cudaSuccess) return e;
+    if (const cudaError_t e = runs_per_sm<NT>(smem, occ)) return e;
     const long long most = (long long)(occ > 0 ? occ : 1) * n_sm;
     k_label_run<NT><<<(unsigned)(A.n_items < most ? A.n_items : most), NT, smem, s>>>(A);
     return cudaGetLastError();
@@ -333,7 +340,30 @@ size_t rid_label_run_smem(int N, int C) {
     return b <= (size_t)RUN_SMEM_MAX ? b : 0;
 }
 
-int rid_label_run_threads(int N) { return N <= 32 ? 128 : N <= 64 ? 256 : 512; }
+// The sizes' times of a wave, in twentieths of the largest's, are those of 80 to 200 beads with every SM full
+// (60 steps of 80 beads, us: 445 for 2 runs an SM at 512 threads, 559 for 4 at 256, 886 for 8 at 128).  By chain
+// length alone -> with the runs, the call's time (and through k_label_fused): 1216 runs of 66 beads 1230 -> 716 us
+// (1061), 4096 of 80 beads 3773 -> 2323 (3570), 1024 of 200 beads 1547 -> 1512 (2280).  608 of 200 beads stay
+// at 512 threads (1056 us, 1128 at 256).
+int rid_label_run_threads(int N, size_t smem, double runs, int n_sm) {
+    const int most = N <= 32 ? 128 : N <= 64 ? 256 : 512;
+    int best = most;
+    double cost = INFINITY;
+    for (int nt = most; nt >= 128; nt /= 2) {
+        int occ = 0;
+        const cudaError_t e = nt == 512 ? runs_per_sm<512>(smem, occ) : nt == 256 ? runs_per_sm<256>(smem, occ)
+                                                                                  : runs_per_sm<128>(smem, occ);
+        if (e != cudaSuccess || occ < 1) continue;
+        const double waves = std::ceil(runs / ((double)occ * n_sm));
+        const double c = waves * (nt == 512 ? 20.0 : nt == 256 ? 25.0 : 39.0);
+        if (c < cost) {
+            cost = c;
+            best = nt;
+        }
+        if (waves <= 1.0) break;   // a smaller size takes longer
+    }
+    return best;
+}
 
 cudaError_t rid_launch_label_run(const FusedArgs& A, int threads, int n_sm, size_t smem, cudaStream_t s) {
     switch (threads) {

@@ -1576,10 +1576,10 @@ extern "C" int rid_label(rid_system* sys, int32_t R, const float* x0, const floa
         int nsm = 1, dev = 0;
         CK(cudaGetDevice(&dev));
         CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-        const int nt = rid_label_run_threads(N);
+        const size_t smem = rid_label_run_smem(N, C);
+        const int nt = rid_label_run_threads(N, smem, R, nsm);
         cudaError_t le = cudaSuccess;
-        TRY(timed_launch(sys, "k_label_run", st,
-                         [&] { le = rid_launch_label_run(A, nt, nsm, rid_label_run_smem(N, C), st); }));
+        TRY(timed_launch(sys, "k_label_run", st, [&] { le = rid_launch_label_run(A, nt, nsm, smem, st); }));
         if (le != cudaSuccess) return fail(RID_ERR_CUDA, "k_label_run launch: %s", cudaGetErrorString(le));
         // the host staging vector must outlive the copy
         CK(cudaStreamSynchronize(st));

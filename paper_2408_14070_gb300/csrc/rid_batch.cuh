@@ -45,10 +45,11 @@ struct FusedArgs {
 // Shared memory for N beads and C CVs, 0 when it does not fit (from about 870
 // beads on):
 size_t rid_label_run_smem(int N, int C);
-// CTA size for a chain of N beads: a warp for every task of a step, up to 16.
-// (More runs than fit at once want it too: 512 uneven runs of 50 to 500 beads
-// took 5.5 ms at 512 threads, 6.4 at 256 and 9.6 at 128.)
-int rid_label_run_threads(int N);
+// CTA size for `runs` runs of chains of up to N beads and smem bytes of shared
+// memory: a warp for every task of a step, up to 16, while that takes as few
+// waves of runs over the SMs; else the smaller size whose waves take least.
+// Runs of different lengths count as many of the longest as they cost.
+int rid_label_run_threads(int N, size_t smem, double runs, int n_sm);
 // threads: 128, 256 or 512; smem: the largest over the items.
 cudaError_t rid_launch_label_run(const FusedArgs& A, int threads, int n_sm, size_t smem, cudaStream_t s);
 

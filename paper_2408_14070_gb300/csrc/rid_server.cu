@@ -1151,8 +1151,9 @@ extern "C" int rid_label_batch(rid_server* srv, const rid_label_job* jobs, int32
     // one's shared memory: classes 0..2 run k_label_run (chains of which one, two,
     // or more fit an SM), class 3 k_label_fused (chains too long for it)
     struct Class {
-        int nt = 0, first = 0, n = 0;
+        int nt = 0, first = 0, n = 0, N = 0;
         size_t smem = 0;
+        double work = 0.0, most = 0.0;   // steps x (beads + 100) of all runs and of the longest
     } cls[4];
     {
         auto class_of = [&](const FusedItem& a) {
@@ -1168,7 +1169,15 @@ extern "C" int rid_label_batch(rid_server* srv, const rid_label_job* jobs, int32
             const size_t b = rid_label_run_smem(S.N, S.C);
             if (!q.n++) q.first = (int)k;
             q.smem = std::max(q.smem, b ? b : rid_label_fused_smem(S.N, S.C, 0));
-            q.nt = threads ? threads : std::max(q.nt, b ? rid_label_run_threads(S.N) : 512);
+            q.N = std::max(q.N, S.N);
+            const double w = (double)jobs[items[k].job].n_steps * (S.N + 100);
+            q.work += w;
+            q.most = std::max(q.most, w);
+        }
+        for (int c = 0; c < 4; ++c) {
+            Class& q = cls[c];
+            if (!q.n) continue;
+            q.nt = threads ? threads : c == 3 ? 512 : rid_label_run_threads(q.N, q.smem, q.work / q.most, srv->n_sm);
         }
     }
     // flag copies for the device path go to a small pinned area instead

@@ -170,3 +170,35 @@ def test_nonfinite_job_is_reported_per_job(R):
     assert np.array_equal(good["mf"], ref["mf"])
     good["system"].close()
     badj["system"].close()
+
+
+@pytest.mark.parametrize("n,runs", [(66, 1216), (80, 640), (200, 456), (24, 1216)])
+def test_many_short_runs_get_a_cta_size_that_holds_them(R, n, runs):
+    # The size chosen (threads = 0) against the fixed ones: 512 threads hold two runs an SM whatever their
+    # length, 1.6 times the time of the best size for 1216 runs of 66 beads.  A quarter more leaves room for the
+    # clock; the bits are those of every size.
+    import time
+    import torch
+    sp = I.make_system(n, 4, 31)
+    x = I.make_chains(8, sp, 31)
+    x0 = torch.from_numpy(np.ascontiguousarray(np.tile(x, (runs // 8, 1, 1)))).cuda()
+    rng = np.random.default_rng(31)
+    s0 = torch.from_numpy(rng.uniform(-1, 1, size=(runs, 4))).cuda()
+    kappa = torch.full((runs, 4), 1.0, dtype=torch.float64, device="cuda")     # (a stiff restraint can make a run non-finite)
+    out = {}
+    t = {}
+    with R.System(sp) as s, R.Server(1 << 30) as srv:
+        for nt in (128, 256, 512, 0):
+            o = [torch.zeros(runs, 4, dtype=torch.float64, device="cuda") for _ in range(3)]
+            job = dict(system=s, x0=x0, v0=None, s0=s0, kappa=kappa, n_steps=100, n_equil=10, n_blocks=5, mf=o[0],
+                       se=o[1], std=o[2])
+            best = 1e9
+            for _ in range(5):
+                torch.cuda.synchronize()
+                t0 = time.perf_counter()
+                srv.label_batch([job], threads=nt)
+                best = min(best, time.perf_counter() - t0)
+            out[nt], t[nt] = torch.stack(o).cpu().numpy(), best
+    for nt in (128, 256, 512):
+        assert np.array_equal(out[nt], out[0]), nt
+    assert t[0] < 1.25 * min(t[128], t[256], t[512]), t
