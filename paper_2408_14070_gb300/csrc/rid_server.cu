@@ -685,9 +685,17 @@ int label_tick_launch(rid_server* srv) {
     A2.items = A.items + n_small;
     A2.n_items = n_big;
     A2.next = reinterpret_cast<int*>(dm + o_cnt + 128);
-    int nt = 256;
+    // CTA sizes: 256 threads for the clusters and for most ticks of short chains.  While two runs an SM hold all
+    // of a tick, its longest chain sets the time, and beyond 288 beads 512 threads take less (a stream of 30 runs x
+    // 1500 steps of 400 beads 27.1 -> 20.3 ms, 150 of 700 beads 43.0 -> 36.3); more than four runs an SM of up
+    // to 128 beads want eight at once (1200 of 50 beads 24.9 -> 18.8 ms).  The same bits at every size.
+    int nt = 256, nt_small = 256, longest = 0;
+    for (int q = 0; q < n_small; ++q) longest = std::max(longest, fj[items[q].job].S.N);
+    if (n_small <= 2 * srv->n_sm) nt_small = longest > 288 ? 512 : 256;
+    else if (n_small > 4 * srv->n_sm && longest <= 128) nt_small = 128;
     const size_t smem_all = std::max(smem, smem_cl);
     if (rid_label_fused_occupancy(nt, smem_all) < 1) nt = 128;
+    if (rid_label_fused_occupancy(nt_small, smem) < 1) nt_small = nt;
     SCK(cudaMemsetAsync(A.next, 0, 256, st));
     SCK(cudaEventRecord(srv->le0, st));
     if (n_big > 0) {
@@ -705,9 +713,9 @@ int label_tick_launch(rid_server* srv) {
         SCK(cudaEventRecord(srv->ljoin, srv->lst2));
     }
     if (n_small > 0) {
-        const int occ = std::max(1, rid_label_fused_occupancy(nt, smem));
+        const int occ = std::max(1, rid_label_fused_occupancy(nt_small, smem));
         const int grid = (int)std::min<long long>(n_small, (long long)occ * srv->n_sm);
-        SCK(rid_launch_label_fused(A, nt, grid, smem, st));
+        SCK(rid_launch_label_fused(A, nt_small, grid, smem, st));
     }
     if (n_big > 0) SCK(cudaStreamWaitEvent(st, srv->ljoin, 0));
     if (!dout.empty()) rid_launch_copy_descs(reinterpret_cast<const CopyDesc*>(dm + o_dout), (int)dout.size(), st);

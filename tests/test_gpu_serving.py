@@ -225,3 +225,24 @@ def test_request_errors(R):
             srv.poll(jid)                          # forgotten after the final status
         small.sys.close()
     big.sys.close()
+
+
+@pytest.mark.parametrize("n,jobs,runs", [
+    (288, 4, 1),        # the longest chain of a tick at 256 threads
+    (289, 4, 1),        # 512 threads
+    (300, 6, 60),       # more than two runs an SM: 256 threads again
+    (128, 12, 60),      # more than four: 128 threads
+    (129, 12, 60),      # a bead too long for them
+])
+def test_ticks_of_every_cta_size_give_the_bits_of_rid_label(R, n, jobs, runs):
+    specs = [Spec(R, "label", n, 5, runs, 80, 40 + k) for k in range(jobs)]
+    for sp in specs:
+        sp.kappa = np.full_like(sp.kappa, 0.5)
+    with R.Server(1 << 30) as srv:
+        ids = [sp.submit(srv) for sp in specs]
+        res = srv.wait(ids)
+    for sp, jid in zip(specs, ids):
+        assert res[jid][0] == R.RID_OK
+        for a, b in zip(sp.outputs(), sp.per_job()):
+            assert np.array_equal(a, b)
+        sp.sys.close()
