@@ -192,10 +192,14 @@ def _check(code: int):
 
 
 # ---------------------------------------------------------------------------
+_WRITEABLE, _WARN_ON_WRITE = 0x400, 0x80000000     # bits of ndarray.flags.num
+
+
 def _host_address(a):
     """Address of a numpy array's first element (the buffer export is several
-    times cheaper than ndarray.ctypes; it needs a writable, non-empty array)."""
-    if a.size and a.flags.writeable:
+    times cheaper than ndarray.ctypes; it needs a writable, non-empty array, and
+    numpy warns when it exports one that broadcast_arrays made)."""
+    if a.size and a.flags.num & (_WRITEABLE | _WARN_ON_WRITE) == _WRITEABLE:
         return C.addressof(C.c_char.from_buffer(a))
     return a.ctypes.data
 
