@@ -40,10 +40,9 @@ struct Smem {
     uint64_t a_full;                 // even CTA: the next operand is complete (epilogue warps of both CTAs)
     uint64_t drain;
     uint32_t tmem_base;
-    int abort_flag;
+    int abort_flag;                  // of this CTA, at the end of either CTA
     int issued;                      // weight iterations whose part this CTA has issued
-    int odd_issued;                  // even CTA: the odd CTA's, and in both CTAs the other one's abort flag
-    int peer_abort;
+    int odd_issued;                  // even CTA: the odd CTA's
 };
 
 constexpr uint32_t PAIR_STAGE = 128u * 128u;   // half of a 256-row weight chunk
@@ -323,7 +322,6 @@ __global__ void __maxnreg__(96)
         S.abort_flag = 0;
         S.issued = 0;
         S.odd_issued = 0;
-        S.peer_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncwarp();
@@ -670,14 +668,13 @@ __global__ void __maxnreg__(96)
         if ((ROWS == 128 || hf == 0) && valid && !S.abort_flag)
             P.Apart[(size_t)m * P.W + wg] = pair_member_value(P, m, tile, row);
     }
-    if (threadIdx.x == 0 && S.abort_flag) {
-        const uint32_t other = rank ^ 1u;
-        st_cluster_u32(mapa(smem_u32(&S.peer_abort), other), 1u);
-    }
-    if (threadIdx.x == 0 && rank == 1) st_cluster_u32(mapa(smem_u32(&S.odd_issued), 0), (uint32_t)S.issued);
+    if (threadIdx.x == 0 && S.abort_flag) st_cluster_u32(mapa(smem_u32(&S.abort_flag), rank ^ 1u), 1u);
     __syncwarp();
     cluster_sync_all();               // no CTA leaves while the pair's MMAs may touch it
-    if (S.abort_flag || S.peer_abort) {   // the same in both CTAs
+    if (S.abort_flag) {               // the same in both CTAs
+        if (threadIdx.x == 0 && rank == 1) st_cluster_u32(mapa(smem_u32(&S.odd_issued), 0), (uint32_t)S.issued);
+        __syncwarp();
+        cluster_sync_all();
         if (rank == 0 && threadIdx.x == 0) land_loads<F8>(P, S);
         __syncwarp();
         cluster_sync_all();           // ... nor while loads that no MMA has waited for are on their way
