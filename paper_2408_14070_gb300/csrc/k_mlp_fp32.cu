@@ -16,8 +16,8 @@
 // into a ring of NSW stages of KC rows in shared memory by cp.async, shared by
 // the eight warps, the first stages of a layer during the epilogue of the one
 // before it.
-// tanh(z_l) of every layer is kept in a global scratch [M][tile][L][H][slots]
-// (L2-resident at the sizes used) for the backward pass:
+// tanh(z_l) of every layer is kept in a global scratch [M][tile][L][H][walkers of
+// the tile] (L2-resident at the sizes used) for the backward pass:
 //   g_L = w_out,  delta_l = g_l * (1 - tanh^2 z_l),
 //   g_{l-1} = W_l^T delta_l (+ g_l for a residual layer),
 //   dA/ds_j = -sin s_j g_0[2j] + cos s_j g_0[2j+1].
@@ -34,6 +34,9 @@ namespace {
 
 constexpr int NT = 256;   // threads per CTA
 constexpr int F32_SMEM_MAX = 227 * 1024;
+
+// Walkers of a member in the scratch, but for groups of seven (choose_rpt).
+__host__ __device__ inline size_t f32_walkers(int W) { return ((size_t)W + 31) / 32 * 32; }
 
 __device__ __forceinline__ void cpa4(float* dst, const float* src, int bytes) {
     const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
@@ -238,12 +241,15 @@ __global__ void __launch_bounds__(NT, RPT >= 4 ? 1 : 2) k_mlp_fp32(MlpF32 E) {
     float* Y = X + (size_t)(BWD && E.resnet ? H : 0) * LD;   // g_l (residual gradient)          [H][LD]
     float* ubuf = Y + (size_t)H * LD;
     float* ws = ubuf + (size_t)D * LD;                  // weight ring [NSW][KC][COLS]
-    const int m = blockIdx.y, tile = blockIdx.x, ntiles = gridDim.x;
-    const int w0 = tile * R;
+    const int m = blockIdx.y, w0 = blockIdx.x * R;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const Lane t = lane_of<WCN>();
-    float* hs = BWD ? E.hs + ((size_t)m * ntiles + tile) * (size_t)L * H * S::SLOTS : nullptr;
     const int own = t.rg * GS;                          // this thread's slots of a row
+    // saved tanh: rows of the tile's slots; a last tile of 64 that holds 32 walkers or fewer keeps half of them
+    const int tw = RPT == 8 && R == 64 && W - w0 <= 32 ? 32 : S::SLOTS;
+    const bool keep = own < tw;
+    const size_t wst = RPT == 7 ? (size_t)gridDim.x * S::SLOTS : f32_walkers(W);
+    float* hs = BWD ? E.hs + (m * wst + (size_t)blockIdx.x * S::SLOTS) * (size_t)L * H + own : nullptr;
 
     // the passes in order: forward layers, then (BWD) gradient layers L - 1 .. 0
     const int npass = BWD ? 2 * L : L;
@@ -313,7 +319,7 @@ __global__ void __launch_bounds__(NT, RPT >= 4 ? 1 : 2) k_mlp_fp32(MlpF32 E) {
                     if constexpr (SPLIT) z += value(acc1, i, j);
                     tv[i] = tanhf(z + bn);
                 }
-                if (BWD) store_group<RPT>(hs + ((size_t)l * H + n) * S::SLOTS + own, tv);
+                if (BWD && keep) store_group<RPT>(hs + ((size_t)l * H + n) * tw, tv);
                 if (E.resnet && l > 0) {
                     load_group<RPT>(X + (size_t)n * LD + own, h);
 #pragma unroll
@@ -338,6 +344,14 @@ __global__ void __launch_bounds__(NT, RPT >= 4 ? 1 : 2) k_mlp_fp32(MlpF32 E) {
         if (lane == 0) E.Aval[(size_t)m * W + w0 + r] = part + E.bout[(long long)m * E.bo_st];
     }
     if constexpr (BWD) {
+        auto load_kept = [&](const float* p, float(&v)[RPT]) {
+            if (keep) {
+                load_group<RPT>(p, v);
+            } else {
+#pragma unroll
+                for (int i = 0; i < RPT; ++i) v[i] = 0.0f;
+            }
+        };
         // ---------------- backward: X holds delta_l, Y g_l of this thread's own columns
         __syncthreads();
 #pragma unroll
@@ -346,7 +360,7 @@ __global__ void __launch_bounds__(NT, RPT >= 4 ? 1 : 2) k_mlp_fp32(MlpF32 E) {
             if (n < H) {
                 const float wn = wo[n];
                 float tv[RPT], g[RPT];
-                load_group<RPT>(hs + ((size_t)(L - 1) * H + n) * S::SLOTS + own, tv);
+                load_kept(hs + ((size_t)(L - 1) * H + n) * tw, tv);
 #pragma unroll
                 for (int i = 0; i < RPT; ++i) {
                     g[i] = wn;
@@ -386,7 +400,7 @@ __global__ void __launch_bounds__(NT, RPT >= 4 ? 1 : 2) k_mlp_fp32(MlpF32 E) {
                     const int n = col_of(t, j);
                     if (n >= H) continue;
                     float v[RPT], tv[RPT];
-                    load_group<RPT>(hs + ((size_t)(l - 1) * H + n) * S::SLOTS + own, tv);
+                    load_kept(hs + ((size_t)(l - 1) * H + n) * tw, tv);
 #pragma unroll
                     for (int i = 0; i < RPT; ++i) v[i] = g[i][j];
                     if (E.resnet) store_group<RPT>(Y + (size_t)n * LD + own, v);
@@ -421,8 +435,11 @@ __global__ void __launch_bounds__(NT, RPT >= 4 ? 1 : 2) k_mlp_fp32(MlpF32 E) {
 // Walkers per thread: the tile whose waves of CTAs over the SMs cost least,
 // counting a K row at the larger of its FMA cycles (16 RPT) and its shared loads
 // (40), plus 8 for what does not overlap; of those that fit in shared memory.
-// Two walkers always fit.
-int choose_rpt(int wcn, int W, int M, int D, int H, int resnet, bool bwd) {
+// Two walkers always fit.  compact: not seven, whose rows of saved tanh are an
+// eighth padding: a server's jobs, whose scratch counts against its budget.  (Rows
+// of seven without padding cost everyone: 4200 -> 4330 us for 20 steps of 1500
+// walkers with 16-, 8- and 4-byte accesses, 4716 with 4-byte ones.)
+int choose_rpt(int wcn, int W, int M, int D, int H, int resnet, bool bwd, bool compact) {
     static int nsm[64] = {};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) dev = 0;
@@ -431,6 +448,7 @@ int choose_rpt(int wcn, int W, int M, int D, int H, int resnet, bool bwd) {
     int best = 2;
     long long cost = -1;
     for (int rpt : {2, 4, 7, 8}) {
+        if (compact && rpt == 7) continue;
         if (tile_smem(rpt, wcn, D, H, resnet, bwd) > (size_t)F32_SMEM_MAX) continue;
         const int R = 2 * (8 / wcn) * rpt;
         const long long ctas = (long long)((W + R - 1) / R) * M;
@@ -635,16 +653,16 @@ static int small_tile(const EnsDev& E, int W) {
     return tw;
 }
 
-// Rounded up over every tile shape (7 walkers take 8 slots), so that it grows
-// with W: a system keeps the scratch of its largest walker count.
-size_t rid_mlp_fp32_scratch_floats(const EnsDev& E, int W) {
-    return (size_t)E.M * E.L * E.H * ((size_t)(W + 27) / 28 * 32 + 64);
+// Rounded up over every tile shape, so that it grows with W: a system keeps the
+// scratch of its largest walker count.  (Groups of seven take eight slots.)
+size_t rid_mlp_fp32_scratch_floats(const EnsDev& E, int W, bool compact) {
+    return (size_t)E.M * E.L * E.H * (compact ? f32_walkers(W) : (size_t)(W + 27) / 28 * 32 + 64);
 }
 
 // The kernel for a width, walkers per thread chosen.
 template <int WCN, bool BWD, bool SPLIT>
 static void launch_shape(const MlpF32& E, int M, cudaStream_t s) {
-    switch (choose_rpt(WCN, E.W, M, E.D, E.H, E.resnet, BWD)) {
+    switch (choose_rpt(WCN, E.W, M, E.D, E.H, E.resnet, BWD, BWD && E.compact)) {
         case 2: return launch_f32<2, WCN, BWD, SPLIT>(E, M, s);
         case 4: return launch_f32<4, WCN, BWD, SPLIT>(E, M, s);
         case 7: return launch_f32<7, WCN, BWD, SPLIT>(E, M, s);
@@ -658,7 +676,7 @@ static void launch_values(const MlpF32& E, int M, cudaStream_t s) {
     else launch_shape<4, false, SPLIT>(E, M, s);
 }
 
-void rid_launch_mlp_fp32(const EnsDev& E, StateDev st, int W, int C, cudaStream_t s, bool values_only) {
+void rid_launch_mlp_fp32(const EnsDev& E, StateDev st, int W, int C, cudaStream_t s, bool values_only, bool compact) {
     if (const int tw = small_tile(E, W)) {
         const SmallLayout Y = small_layout(E.D, E.L, E.H, E.resnet, tw);
         const int wpt = (tw + NT / E.H - 1) / (NT / E.H);
@@ -695,6 +713,7 @@ void rid_launch_mlp_fp32(const EnsDev& E, StateDev st, int W, int C, cudaStream_
     A.W = W;
     A.C = C;
     A.hs = st.hs;
+    A.compact = compact;
     A.Aval = st.Aval;
     A.gradA = st.gradA;
     A.cvdist = E.cvdist;

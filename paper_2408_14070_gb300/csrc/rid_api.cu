@@ -234,7 +234,7 @@ static int ensure_state(rid_system* sys, int W) {
         TRY(sys->Aval.ensure((size_t)E.M * W * sizeof(float)));
         TRY(sys->Aval.ensure((size_t)E.M * W * sizeof(float)));
         if (sys->precision == RID_PREC_FP32) {
-            TRY(sys->hs.ensure(rid_mlp_fp32_scratch_floats(E, W) * sizeof(float)));
+            TRY(sys->hs.ensure(rid_mlp_fp32_scratch_floats(E, W, sys->serving) * sizeof(float)));
         } else {
             const size_t ntiles = rid_tc_tiles(W);
             TRY(sys->tsave.ensure((size_t)E.M * ntiles * E.L * 128 * E.H * sizeof(__nv_bfloat16)));
@@ -1021,7 +1021,10 @@ static int launch_mlp(rid_system* sys, int W, int mode, StateDev sd, cudaStream_
         E.aslices = 1;
     } else if (mode == 1) {
         E.aslices = 1;
-        TRY(timed_launch(sys, "k_mlp_fp32", st, [&] { rid_launch_mlp_fp32(E, sd, W, sys->S.C, st, values_only); }));
+        // (the scratch may be a served job's, also when the walkers are advanced directly later)
+        const bool compact = sys->hs.bytes < rid_mlp_fp32_scratch_floats(E, W, false) * sizeof(float);
+        TRY(timed_launch(sys, "k_mlp_fp32", st,
+                         [&] { rid_launch_mlp_fp32(E, sd, W, sys->S.C, st, values_only, compact); }));
     }
     return RID_OK;
 }
@@ -1365,7 +1368,7 @@ size_t rid_sys_footprint(const rid_system* sys, int W) {
     if (sys->has_ens) {
         const EnsDev& E = sys->E;
         b += (size_t)E.M * nc * 4 + (size_t)E.M * W * 4;
-        if (sys->precision == RID_PREC_FP32) b += rid_mlp_fp32_scratch_floats(E, W) * 4;
+        if (sys->precision == RID_PREC_FP32) b += rid_mlp_fp32_scratch_floats(E, W, true) * 4;   // (its jobs run compact)
         else b += (size_t)E.M * rid_tc_tiles(W) * 128 * (E.H * (E.L * 2 + (E.resnet ? 4 : 0)) + TC_MAX_QSLICES * 4);
     }
     return b;

@@ -327,14 +327,15 @@ struct MlpF32 {
     long long wo_st, bo_st;
     const float* u;          // [W][D]
     int D, L, H, resnet, W, C;
-    float* hs;               // rid_mlp_fp32_scratch_floats (input gradient only)
+    float* hs;               // rid_mlp_fp32_scratch_floats (input gradient only), of its compact form if
+    bool compact;            // this is set
     float* Aval;             // [M][W]
     float* gradA;            // [M][W][C]
     const int* cvdist;
 };
 // values_only: the member values may be formed without the input gradient
-void rid_launch_mlp_fp32(const EnsDev& E, StateDev st, int W, int C, cudaStream_t s, bool values_only = false);
-size_t rid_mlp_fp32_scratch_floats(const EnsDev& E, int W);
+void rid_launch_mlp_fp32(const EnsDev& E, StateDev st, int W, int C, cudaStream_t s, bool values_only, bool compact);
+size_t rid_mlp_fp32_scratch_floats(const EnsDev& E, int W, bool compact);
 // Member values alone; split sums the K tiles of 32 with even and odd index apart
 // (the order of MCMC batches below 1024 walkers or 64 columns).
 void rid_launch_mlp_values(const MlpF32& E, int M, bool split, cudaStream_t s);

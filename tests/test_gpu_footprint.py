@@ -23,7 +23,7 @@ def R():
 def _needed(R, sysobj, x0, steps):
     with R.Server(1 << 20) as srv:            # the smallest budget
         with pytest.raises(R.RidError) as e:
-            srv.submit_explore(sysobj, x0, steps, x_out=np.zeros_like(x0))
+            srv.cancel(srv.submit_explore(sysobj, x0, steps, x_out=np.zeros_like(x0)))
     return int(re.search(r"needs (\d+) bytes", str(e.value))[1])
 
 
@@ -49,3 +49,13 @@ def test_tensor_core_scratch_is_counted_in_tiles_of_128_walkers(R, prec, W, H, r
     with R.System(sp) as s:
         s.set_ensemble(ens, precision={"bf16": R.RID_PREC_BF16, "fp8": R.RID_PREC_FP8}[prec])
         assert _needed(R, s, x0, 20) <= _bound(sp, ens, W, prec, resnet, 20)
+
+
+@pytest.mark.parametrize("W,H,resnet", [(12, 300, True), (33, 256, False), (1000, 128, False), (1999, 256, True)])
+def test_fp32_scratch_is_counted_for_the_walkers_of_the_call(R, W, H, resnet):
+    sp = I.make_system(30, 6, 3, output_freq=10)
+    ens = I.make_ensemble(16, 12, 4, H, 3, resnet=resnet)
+    x0 = I.make_chains(W, sp, 3)
+    with R.System(sp) as s:
+        s.set_ensemble(ens, precision=R.RID_PREC_FP32)
+        assert _needed(R, s, x0, 20) <= _bound(sp, ens, W, "fp32", resnet, 20)
