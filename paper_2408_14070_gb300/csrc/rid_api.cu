@@ -996,7 +996,10 @@ static int launch_mlp(rid_system* sys, int W, int mode, StateDev sd, cudaStream_
             E.aslices = 1;
             return RID_OK;
         }
-        const int cs = sys->cs_force ? sys->cs_force : V.cs_W == W ? V.csize : default_cluster(P.ntiles * E.M);
+        // (the tuner's size is one for the force field beside the ensemble; nothing runs beside member values)
+        const int cs = sys->cs_force                 ? sys->cs_force
+                       : V.cs_W == W && !values_only ? V.csize
+                                                     : default_cluster(P.ntiles * E.M);
         if (sys->cs_force > 1 && !V.cl_ok[cs == 2 ? 1 : 2])
             return fail(RID_ERR_ARG, "ensemble kernel: cluster size %d does not fit this ensemble's shape", cs);
         sys->tcv.used_cs = cs;

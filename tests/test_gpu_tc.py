@@ -418,3 +418,31 @@ def test_full_size_as_benched(R, orc):
         assert np.abs(np.angle(np.exp(1j * (cv[w, -1] - sr)))).max() < 1e-4, w
         e = orc.ensemble(ens, sr)
         assert abs(et[w, -1] - e["eps"]) <= EPS_TOL * abs(e["eps"]) + 1e-4, w
+
+
+def test_member_values_take_the_size_for_a_launch_alone(R):
+    # 1024 walkers of 200 beads: the tuner weighs the ensemble against the force field beside it and keeps size 1
+    # there.  Member values have nothing beside them: pairs of 64 rows while they fit the SMs at once, also on a
+    # system that has explored as many walkers.
+    W = 1024
+    sp = I.make_system(200, 20, 3, output_freq=5)
+    ens = I.make_ensemble(4, 40, 4, 256, 3)
+    x0 = np.ascontiguousarray(np.tile(I.make_chains(8, sp, 3), (W // 8, 1, 1)))
+    s0 = np.random.default_rng(3).uniform(-3, 3, (W, 20)).astype(np.float32)
+    out = [np.zeros_like(s0) for _ in range(3)]
+    with R.System(sp) as fresh, R.System(sp) as explored:
+        for s in (fresh, explored):
+            s.set_ensemble(ens, precision=R.RID_PREC_BF16)
+        explored.explore(x0, 5, x_out=np.zeros_like(x0))
+        tuned = explored.mlp_cluster()
+        for s, o in zip((fresh, explored), out):
+            s.mcmc(s0, 3, 0, 1.0, 0.2, 7, bins=21, s_out=o)
+        print(f"\nexplored at size {tuned}, member values at {explored.mlp_cluster()}")
+        assert fresh.mlp_cluster() == explored.mlp_cluster() == 2
+        # the exploration's size is still the tuned one, and a pinned size holds for member values too
+        explored.explore(x0, 5, x_out=np.zeros_like(x0))
+        assert explored.mlp_cluster() == tuned
+        explored.set_mlp_cluster(1)
+        explored.mcmc(s0, 3, 0, 1.0, 0.2, 7, bins=21, s_out=out[2])
+        assert explored.mlp_cluster() == 1
+    assert np.array_equal(out[0], out[1]) and np.array_equal(out[0], out[2])
