@@ -7,7 +7,8 @@
 // its inputs.  In a warp, half (lane / 16) takes one group of RPT walkers and
 // lane % 16 the columns 4 lc .. + 3 and 64 + 4 lc .. + 3, so a thread keeps an
 // RPT x 8 register tile, accumulated by fma.rn.f32x2 (two neighbouring columns
-// an instruction; each half rounds as fmaf does).  Activations live in shared
+// an instruction; each half rounds as fmaf does).  (Member values of widths to 64
+// and 32 take CPT = 4 and 2 columns a thread, 16 CPT a warp.)  Activations live in shared
 // memory transposed as [neuron][walker] rows of LD floats, one group of RPT
 // walkers in GS slots (RPT rounded up to a power of two), so a thread's walkers
 // are one or two 16-byte loads; a layer's outputs go back over its inputs once
@@ -28,6 +29,8 @@
 // 1024 walkers x 4 members 40-256x4-1 (128 tiles of 32): 238 us with a 256-thread
 // CTA of 8 x 4 register tiles, scalar FMAs and 8-row stages, 115 us now (29.5 of
 // 69.8 TFLOP/s); a force evaluation of them 353 -> 237 us.
+#include <algorithm>
+
 #include "rid_internal.cuh"
 
 namespace {
@@ -64,15 +67,15 @@ __device__ __forceinline__ void fma2(f32x2& acc, f32x2 a, f32x2 b) {
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
 }
 
-// Tile shape: RPT walkers a thread, WCN warp columns.
-template <int RPT, int WCN>
+// Tile shape: RPT walkers and CPT columns a thread, WCN warp columns.
+template <int RPT, int WCN, int CPT>
 struct Shape {
     static constexpr int GS = RPT > 4 ? 8 : RPT > 2 ? 4 : RPT;   // slots of a walker group
     static constexpr int GROUPS = 2 * (8 / WCN);                 // walker groups of a CTA
     static constexpr int R = GROUPS * RPT;                       // walkers of a CTA
     static constexpr int SLOTS = GROUPS * GS;
     static constexpr int LD = SLOTS + 4;                         // floats of a shared row
-    static constexpr int COLS = 128 * WCN;                       // output neurons
+    static constexpr int COLS = 16 * CPT * WCN;                  // output neurons
     // weight rows per ring stage: 32 KB a stage (16 rows of 256 columns cost 84 us where 32 cost
     // 78, for twice the block barriers); short tiles, whose rows are consumed faster than one
     // stage ahead arrives, keep more stages
@@ -83,10 +86,10 @@ __host__ __device__ constexpr int shape_gs(int rpt) { return rpt > 4 ? 8 : rpt >
 
 // Shared memory of a tile, bytes: activations (and, for a residual gradient, g_l
 // beside them), the inputs, the weight ring.
-size_t tile_smem(int rpt, int wcn, int D, int H, int resnet, bool bwd) {
+size_t tile_smem(int rpt, int wcn, int cpt, int D, int H, int resnet, bool bwd) {
     const int slots = 2 * (8 / wcn) * shape_gs(rpt), ld = slots + 4;
     const int kc = wcn == 4 ? 16 : 32, nsw = rpt <= 2 ? 4 : 2;
-    return sizeof(float) * ((size_t)(bwd && resnet ? 2 : 1) * H * ld + (size_t)D * ld + (size_t)nsw * kc * 128 * wcn);
+    return sizeof(float) * ((size_t)(bwd && resnet ? 2 : 1) * H * ld + (size_t)D * ld + (size_t)nsw * kc * 16 * cpt * wcn);
 }
 
 // Where a thread's outputs lie: walker group, column base of its warp.
@@ -98,9 +101,11 @@ __device__ __forceinline__ Lane lane_of() {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     return Lane{(warp / WCN) * 2 + (lane >> 4), lane & 15, warp % WCN};
 }
-// Column j (0..7) of a thread within a pass.
+// Column j (0 .. CPT - 1) of a thread within a pass.
+template <int CPT>
 __device__ __forceinline__ int col_of(const Lane& t, int j) {
-    return 128 * t.wc + (j < 4 ? 4 * t.lc + j : 64 + 4 * t.lc + j - 4);
+    if (CPT == 2) return 32 * t.wc + 2 * t.lc + j;
+    return 16 * CPT * t.wc + (j < 4 ? 4 * t.lc + j : 64 + 4 * t.lc + j - 4);
 }
 
 // The RPT values of a walker group at p (GS slots, aligned to them).
@@ -181,29 +186,36 @@ __device__ __forceinline__ void ring_prime(const Stream& q, float* ws) {
 // accumulator over k in increasing order.  SPLIT sums the K tiles of 32 with
 // even and odd index in acc and acc1.  Ends with every warp past its last read
 // of `in` and of the ring.
-template <int RPT, int WCN, bool SPLIT>
-__device__ __forceinline__ void tile_gemm(const float* in, const Stream& q, const Lane& t, f32x2 (&acc)[RPT][4],
-                                          f32x2 (&acc1)[SPLIT ? RPT : 1][4], float* ws) {
-    using S = Shape<RPT, WCN>;
+template <int RPT, int WCN, int CPT, bool SPLIT>
+__device__ __forceinline__ void tile_gemm(const float* in, const Stream& q, const Lane& t, f32x2 (&acc)[RPT][CPT / 2],
+                                          f32x2 (&acc1)[SPLIT ? RPT : 1][CPT / 2], float* ws) {
+    using S = Shape<RPT, WCN, CPT>;
     constexpr int KC = S::KC, COLS = S::COLS, NSW = S::NSW;
     const int nst = (q.K + KC - 1) / KC;
-    const bool use = 128 * t.wc < q.nuse;    // warp-uniform: some column of this warp is wanted
-    auto stage = [&](int st, f32x2(&a)[RPT][4]) {
-        const float* wsr = ws + (st % NSW) * KC * COLS + 128 * t.wc + 4 * t.lc;
+    const bool use = 16 * CPT * t.wc < q.nuse;    // warp-uniform: some column of this warp is wanted
+    auto stage = [&](int st, f32x2(&a)[RPT][CPT / 2]) {
+        const float* wsr = ws + (st % NSW) * KC * COLS + 16 * CPT * t.wc + (CPT == 2 ? 2 : 4) * t.lc;
         const float* ar = in + (size_t)st * KC * S::LD + t.rg * S::GS;
         const int kn = q.K - st * KC < KC ? q.K - st * KC : KC;
         auto row = [&](int r) {
             float av[RPT];
             load_group<RPT>(ar + r * S::LD, av);
-            const ulonglong2 w0 = *reinterpret_cast<const ulonglong2*>(wsr + r * COLS);
-            const ulonglong2 w1 = *reinterpret_cast<const ulonglong2*>(wsr + r * COLS + 64);
+            f32x2 w[CPT / 2];
+            if constexpr (CPT == 2) {
+                w[0] = *reinterpret_cast<const f32x2*>(wsr + r * COLS);
+            } else {
+#pragma unroll
+                for (int h = 0; h < CPT / 4; ++h) {
+                    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(wsr + r * COLS + 64 * h);
+                    w[2 * h] = v.x;
+                    w[2 * h + 1] = v.y;
+                }
+            }
 #pragma unroll
             for (int i = 0; i < RPT; ++i) {
                 const f32x2 d = pack2(av[i], av[i]);
-                fma2(a[i][0], d, w0.x);
-                fma2(a[i][1], d, w0.y);
-                fma2(a[i][2], d, w1.x);
-                fma2(a[i][3], d, w1.y);
+#pragma unroll
+                for (int h = 0; h < CPT / 2; ++h) fma2(a[i][h], d, w[h]);
             }
         };
         if (kn == KC) {
@@ -231,9 +243,10 @@ __device__ __forceinline__ void tile_gemm(const float* in, const Stream& q, cons
 }
 
 // BWD: the input gradient as well; else the member values alone.
-template <int RPT, int WCN, bool BWD, bool SPLIT>
-__global__ void __launch_bounds__(NT, RPT >= 4 ? 1 : 2) k_mlp_fp32(MlpF32 E) {
-    using S = Shape<RPT, WCN>;
+template <int RPT, int WCN, int CPT, bool BWD, bool SPLIT>
+__global__ void __launch_bounds__(NT, RPT >= 4 && CPT == 8 ? 1 : 2) k_mlp_fp32(MlpF32 E) {
+    static_assert(CPT == 8 || !BWD, "the input gradient takes eight columns a thread");
+    using S = Shape<RPT, WCN, CPT>;
     constexpr int GS = S::GS, LD = S::LD, R = S::R;
     extern __shared__ __align__(16) float sm[];
     const int D = E.D, L = E.L, H = E.H, W = E.W;
@@ -285,9 +298,9 @@ __global__ void __launch_bounds__(NT, RPT >= 4 ? 1 : 2) k_mlp_fp32(MlpF32 E) {
     }
     __syncthreads();
 
-    f32x2 acc1[SPLIT ? RPT : 1][4];
+    f32x2 acc1[SPLIT ? RPT : 1][CPT / 2];
     // value (i, j) of an accumulator set
-    auto value = [](const f32x2(&a)[RPT][4], int i, int j) {
+    auto value = [](const f32x2(&a)[RPT][CPT / 2], int i, int j) {
         float lo, hi;
         unpack2(a[i][j >> 1], lo, hi);
         return (j & 1) ? hi : lo;
@@ -295,21 +308,21 @@ __global__ void __launch_bounds__(NT, RPT >= 4 ? 1 : 2) k_mlp_fp32(MlpF32 E) {
     // ---------------- forward
     for (int l = 0; l < L; ++l) {
         const float* bias = E.b + (long long)m * E.b_st + E.boff[l];
-        f32x2 acc[RPT][4];
+        f32x2 acc[RPT][CPT / 2];
 #pragma unroll
         for (int i = 0; i < RPT; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+            for (int j = 0; j < CPT / 2; ++j) acc[i][j] = 0ull;
         if constexpr (SPLIT)
 #pragma unroll
             for (int i = 0; i < RPT; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc1[i][j] = 0ull;
-        tile_gemm<RPT, WCN, SPLIT>(l == 0 ? ubuf : X, cur, t, acc, acc1, ws);
+                for (int j = 0; j < CPT / 2; ++j) acc1[i][j] = 0ull;
+        tile_gemm<RPT, WCN, CPT, SPLIT>(l == 0 ? ubuf : X, cur, t, acc, acc1, ws);
         next_pass();
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int n = col_of(t, j);
+        for (int j = 0; j < CPT; ++j) {
+            const int n = col_of<CPT>(t, j);
             if (n < H) {
                 const float bn = bias[n];
                 float tv[RPT], h[RPT];
@@ -356,7 +369,7 @@ __global__ void __launch_bounds__(NT, RPT >= 4 ? 1 : 2) k_mlp_fp32(MlpF32 E) {
         __syncthreads();
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            const int n = col_of(t, j);
+            const int n = col_of<8>(t, j);
             if (n < H) {
                 const float wn = wo[n];
                 float tv[RPT], g[RPT];
@@ -377,7 +390,7 @@ __global__ void __launch_bounds__(NT, RPT >= 4 ? 1 : 2) k_mlp_fp32(MlpF32 E) {
             float g[RPT][8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                const int n = col_of(t, j);
+                const int n = col_of<8>(t, j);
                 float v[RPT];
                 if (res && n < H) load_group<RPT>(Y + (size_t)n * LD + own, v);
 #pragma unroll
@@ -387,7 +400,7 @@ __global__ void __launch_bounds__(NT, RPT >= 4 ? 1 : 2) k_mlp_fp32(MlpF32 E) {
             for (int i = 0; i < RPT; ++i)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) acc[i][j] = pack2(g[i][2 * j], g[i][2 * j + 1]);
-            tile_gemm<RPT, WCN, false>(X, cur, t, acc, acc1, ws);
+            tile_gemm<RPT, WCN, CPT, false>(X, cur, t, acc, acc1, ws);
             next_pass();
 #pragma unroll
             for (int i = 0; i < RPT; ++i)
@@ -397,7 +410,7 @@ __global__ void __launch_bounds__(NT, RPT >= 4 ? 1 : 2) k_mlp_fp32(MlpF32 E) {
                 // g_{l-1}, and its delta over delta_l
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    const int n = col_of(t, j);
+                    const int n = col_of<8>(t, j);
                     if (n >= H) continue;
                     float v[RPT], tv[RPT];
                     load_kept(hs + ((size_t)(l - 1) * H + n) * tw, tv);
@@ -413,7 +426,7 @@ __global__ void __launch_bounds__(NT, RPT >= 4 ? 1 : 2) k_mlp_fp32(MlpF32 E) {
                 // dA/ds_j = -sin s_j g0[2j] + cos s_j g0[2j+1] (torsion), g0[2j] (distance: input (s, 0))
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    const int n = col_of(t, 2 * q), j = n >> 1;
+                    const int n = col_of<8>(t, 2 * q), j = n >> 1;
                     if (n >= D) continue;
                     const bool dist = E.cvdist && __ldg(E.cvdist + j);
                     float cs[RPT], sn[RPT];
@@ -439,7 +452,7 @@ __global__ void __launch_bounds__(NT, RPT >= 4 ? 1 : 2) k_mlp_fp32(MlpF32 E) {
 // eighth padding: a server's jobs, whose scratch counts against its budget.  (Rows
 // of seven without padding cost everyone: 4200 -> 4330 us for 20 steps of 1500
 // walkers with 16-, 8- and 4-byte accesses, 4716 with 4-byte ones.)
-int choose_rpt(int wcn, int W, int M, int D, int H, int resnet, bool bwd, bool compact) {
+int choose_rpt(int wcn, int cpt, int W, int M, int D, int H, int resnet, bool bwd, bool compact) {
     static int nsm[64] = {};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) dev = 0;
@@ -449,10 +462,10 @@ int choose_rpt(int wcn, int W, int M, int D, int H, int resnet, bool bwd, bool c
     long long cost = -1;
     for (int rpt : {2, 4, 7, 8}) {
         if (compact && rpt == 7) continue;
-        if (tile_smem(rpt, wcn, D, H, resnet, bwd) > (size_t)F32_SMEM_MAX) continue;
+        if (tile_smem(rpt, wcn, cpt, D, H, resnet, bwd) > (size_t)F32_SMEM_MAX) continue;
         const int R = 2 * (8 / wcn) * rpt;
         const long long ctas = (long long)((W + R - 1) / R) * M;
-        const long long c = (ctas + n - 1) / n * ((16 * rpt > 40 ? 16 * rpt : 40) + 8);
+        const long long c = (ctas + n - 1) / n * (std::max(2 * cpt * rpt, 40) + 8);
         if (cost < 0 || c <= cost) {
             cost = c;
             best = rpt;
@@ -461,13 +474,13 @@ int choose_rpt(int wcn, int W, int M, int D, int H, int resnet, bool bwd, bool c
     return best;
 }
 
-template <int RPT, int WCN, bool BWD, bool SPLIT>
+template <int RPT, int WCN, int CPT, bool BWD, bool SPLIT>
 void launch_f32(const MlpF32& E, int M, cudaStream_t s) {
     static RidOnce once;
-    auto k = k_mlp_fp32<RPT, WCN, BWD, SPLIT>;
+    auto k = k_mlp_fp32<RPT, WCN, CPT, BWD, SPLIT>;
     rid_opt_in(once, F32_SMEM_MAX, k);
-    constexpr int R = Shape<RPT, WCN>::R;
-    k<<<dim3((E.W + R - 1) / R, M), NT, tile_smem(RPT, WCN, E.D, E.H, E.resnet, BWD), s>>>(E);
+    constexpr int R = Shape<RPT, WCN, CPT>::R;
+    k<<<dim3((E.W + R - 1) / R, M), NT, tile_smem(RPT, WCN, CPT, E.D, E.H, E.resnet, BWD), s>>>(E);
 }
 
 // Small ensembles (every layer of a member fits in shared memory at once, as
@@ -660,20 +673,25 @@ size_t rid_mlp_fp32_scratch_floats(const EnsDev& E, int W, bool compact) {
 }
 
 // The kernel for a width, walkers per thread chosen.
-template <int WCN, bool BWD, bool SPLIT>
+template <int WCN, int CPT, bool BWD, bool SPLIT>
 static void launch_shape(const MlpF32& E, int M, cudaStream_t s) {
-    switch (choose_rpt(WCN, E.W, M, E.D, E.H, E.resnet, BWD, BWD && E.compact)) {
-        case 2: return launch_f32<2, WCN, BWD, SPLIT>(E, M, s);
-        case 4: return launch_f32<4, WCN, BWD, SPLIT>(E, M, s);
-        case 7: return launch_f32<7, WCN, BWD, SPLIT>(E, M, s);
-        default: return launch_f32<8, WCN, BWD, SPLIT>(E, M, s);
+    switch (choose_rpt(WCN, CPT, E.W, M, E.D, E.H, E.resnet, BWD, BWD && E.compact)) {
+        case 2: return launch_f32<2, WCN, CPT, BWD, SPLIT>(E, M, s);
+        case 4: return launch_f32<4, WCN, CPT, BWD, SPLIT>(E, M, s);
+        case 7: return launch_f32<7, WCN, CPT, BWD, SPLIT>(E, M, s);
+        default: return launch_f32<8, WCN, CPT, BWD, SPLIT>(E, M, s);
     }
 }
+// (Widths to 32 and 64 with eight columns a thread, three quarters or half of them for nothing: 20 steps of 100000
+// walkers of 4 x 40-32x4-1 13.7 ms, 6.4 with two; 20000 walkers at width 64 4.16 -> 2.65 ms.  One GEMM a layer, as
+// it was before, took 10.1 and 4.09 ms.)
 template <bool SPLIT>
 static void launch_values(const MlpF32& E, int M, cudaStream_t s) {
-    if (E.H <= 128) launch_shape<1, false, SPLIT>(E, M, s);
-    else if (E.H <= 256) launch_shape<2, false, SPLIT>(E, M, s);
-    else launch_shape<4, false, SPLIT>(E, M, s);
+    if (E.H <= 32) launch_shape<1, 2, false, SPLIT>(E, M, s);
+    else if (E.H <= 64) launch_shape<1, 4, false, SPLIT>(E, M, s);
+    else if (E.H <= 128) launch_shape<1, 8, false, SPLIT>(E, M, s);
+    else if (E.H <= 256) launch_shape<2, 8, false, SPLIT>(E, M, s);
+    else launch_shape<4, 8, false, SPLIT>(E, M, s);
 }
 
 void rid_launch_mlp_fp32(const EnsDev& E, StateDev st, int W, int C, cudaStream_t s, bool values_only, bool compact) {
@@ -718,8 +736,8 @@ void rid_launch_mlp_fp32(const EnsDev& E, StateDev st, int W, int C, cudaStream_
     A.gradA = st.gradA;
     A.cvdist = E.cvdist;
     if (values_only) launch_values<false>(A, E.M, s);
-    else if (E.H <= 256) launch_shape<2, true, false>(A, E.M, s);
-    else launch_shape<4, true, false>(A, E.M, s);
+    else if (E.H <= 256) launch_shape<2, 8, true, false>(A, E.M, s);
+    else launch_shape<4, 8, true, false>(A, E.M, s);
 }
 
 void rid_launch_mlp_values(const MlpF32& E, int M, bool split, cudaStream_t s) {

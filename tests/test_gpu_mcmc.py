@@ -384,3 +384,45 @@ def test_system_with_distance_cvs_on_the_tensor_cores(R, prec):
     assert 0 < nacc < W * K
     for c in np.flatnonzero(dist):
         assert np.all((s[:, c] >= lo[c]) & (s[:, c] <= hi[c]))
+
+
+def _embedded(w, C, L, H, wide):
+    """The packed member w with hidden units of zero weights up to `wide`."""
+    D, p, out, fin, finw = 2 * C, 0, [], 2 * C, 2 * C
+    for _ in range(L):
+        a = np.zeros((wide, finw), np.float32)
+        a[:H, :fin] = w[p:p + H * fin].reshape(H, fin)
+        p += H * fin
+        b = np.zeros(wide, np.float32)
+        b[:H] = w[p:p + H]
+        p += H
+        out += [a.ravel(), b]
+        fin, finw = H, wide
+    o = np.zeros(wide + 1, np.float32)
+    o[:H], o[wide] = w[p:p + H], w[p + H]
+    return np.concatenate(out + [o])
+
+
+@pytest.mark.parametrize("H,W,C,L,resnet", [
+    (5, 1, 2, 1, False),         # one walker, one layer
+    (16, 37, 3, 2, False),
+    (32, 900, 20, 3, True),      # two columns a thread, all of them
+    (33, 500, 20, 3, False),     # four columns a thread: the first width
+    (64, 1023, 20, 4, True),     # all of them, sums split over K
+    (64, 3000, 20, 2, False),    # ... and not
+    (32, 3000, 16, 4, False),
+])
+def test_narrow_networks_give_the_bits_of_the_wide_kernel(R, H, W, C, L, resnet):
+    # Widths to 32 and 64 keep two and four columns a thread, the same network with units of zero weights at
+    # width 96 eight: every sum gains exact zeros only, so the walks agree in every bit.
+    ens = I.make_ensemble(3, 2 * C, L, H, H + W, resnet=resnet)
+    wide = np.stack([_embedded(w, C, L, H, 96) for w in ens.weights])
+    s0 = np.random.default_rng(W).uniform(-3, 3, (W, C)).astype(np.float32)
+    res = []
+    for w, width in ((ens.weights, H), (wide, 96)):
+        s, h1 = np.zeros_like(s0), np.zeros((C, 31), np.uint64)
+        n = R.mcmc(w, 3, C, L, width, s0, 6, 1, 1.0, 0.3, 5, bins=31, resnet=resnet, s_out=s, hist1=h1)
+        res.append((n, s, h1))
+    assert res[0][0] == res[1][0] and 0 < res[0][0]
+    np.testing.assert_array_equal(res[0][1], res[1][1])
+    np.testing.assert_array_equal(res[0][2], res[1][2])
