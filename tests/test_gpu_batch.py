@@ -202,3 +202,44 @@ def test_many_short_runs_get_a_cta_size_that_holds_them(R, n, runs):
     for nt in (128, 256, 512):
         assert np.array_equal(out[nt], out[0]), nt
     assert t[0] < 1.25 * min(t[128], t[256], t[512]), t
+
+
+@pytest.mark.parametrize("dense", [False, True])
+@pytest.mark.parametrize("n,C", [
+    (744, 20),          # the last lists of full length in one CTA's shared memory
+    (768, 20),          # shortened lists from here on; rid_label takes the per-step kernels
+    (1000, 20),         # lists of 24 entries
+    (1024, 20),
+    (1020, 128),        # the shortest lists, 16 entries
+    (1024, 128),        # too long for them: the kernel of longer chains
+])
+def test_short_lists_give_the_bits_of_the_per_step_kernels(R, n, C, dense):
+    # dense: folded on a lattice, so that rows hold more neighbours than a list and the others change them (bonds
+    # and pairs only: a straight chain's angles and dihedrals are singular); far-apart torsions as CVs
+    sp = I.make_system(n, C, 3, **(dict(angle_k=0.0) if dense else {}))
+    rng = np.random.default_rng(n + C)
+    if dense:
+        sp.dihedral_k[:] = 0.0
+        sp.cv_atoms[:] = np.sort(rng.permuted(np.tile(np.arange(n), (C, 1)), axis=1)[:, :4], axis=1)
+        side = int(np.ceil(n ** (1 / 3)))
+        k = np.arange(n)
+        z, y, x = k // side ** 2, k // side % side, k % side
+        y = np.where(z % 2, side - 1 - y, y)
+        x = np.where((z * side + k // side % side) % 2, side - 1 - x, x)
+        x0 = (1.15 * np.stack([x, y, z], -1) + rng.uniform(-0.05, 0.05, (2, n, 3))).astype(np.float32)
+    else:
+        x0 = I.make_chains(2, sp, 3)
+    v0 = rng.standard_normal(x0.shape).astype(np.float32)
+    s0, kappa = rng.uniform(-1, 1, size=(2, C)), np.full((2, C), 0.5)
+    sysobj = R.System(sp)
+    j = dict(system=sysobj, x0=x0, v0=v0, s0=s0, kappa=kappa, step0=0, n_steps=30, n_equil=3, n_blocks=3,
+             mf=np.zeros((2, C)), se=np.zeros((2, C)), std=np.zeros((2, C)), x_out=np.zeros_like(x0),
+             v_out=np.zeros_like(x0))
+    sysobj.set_fused_steps(False)
+    ref = alone(j)
+    with R.Server(64 << 20) as srv:
+        for threads in (0, 128):
+            srv.label_batch([j], threads=threads)
+            for key in ("mf", "se", "std", "x_out", "v_out"):
+                assert np.array_equal(j[key], ref[key]), (threads, key)
+    sysobj.close()

@@ -446,3 +446,44 @@ def test_member_values_take_the_size_for_a_launch_alone(R):
         explored.mcmc(s0, 3, 0, 1.0, 0.2, 7, bins=21, s_out=out[2])
         assert explored.mlp_cluster() == 1
     assert np.array_equal(out[0], out[1]) and np.array_equal(out[0], out[2])
+
+
+def test_pairs_of_several_systems_on_their_own_streams(R):
+    # CTAs of different systems' ensemble kernels meet on the SMs, with 64 to 512 columns of tensor memory each:
+    # pairs of both sizes, one-tile CTAs and the small-batch clusters.  Every call gives the bits it gives alone.
+    import threading
+    import torch
+    shapes = [(300, 64, False), (600, 512, False), (300, 256, True), (100, 192, False), (700, 160, False), (12, 300, True)]
+    systems, x0s, alone = [], [], []
+    for k, (W, H, resnet) in enumerate(shapes):
+        sp = I.make_system(40, 6, 3 + k, output_freq=5)
+        s = R.System(sp)
+        s.set_ensemble(I.make_ensemble(4, 12, 3, H, 3 + k, resnet=resnet), precision=R.RID_PREC_BF16)
+        x0s.append(torch.from_numpy(I.make_chains(W, sp, 3 + k)).cuda())
+        systems.append(s)
+        out = torch.zeros_like(x0s[-1])
+        s.explore(x0s[-1], 40, x_out=out)
+        torch.cuda.synchronize()
+        alone.append(out.clone())
+    got = [[torch.zeros_like(x) for _ in range(4)] for x in x0s]
+    errors, start = [], threading.Barrier(len(shapes))
+
+    def go(k):
+        try:
+            st = torch.cuda.Stream()
+            start.wait()
+            for o in got[k]:
+                systems[k].explore(x0s[k], 40, x_out=o, stream=st)
+            st.synchronize()
+        except Exception as e:      # reported by the main thread
+            errors.append(repr(e))
+
+    threads = [threading.Thread(target=go, args=(k,)) for k in range(len(shapes))]
+    torch.cuda.synchronize()
+    [t.start() for t in threads]
+    [t.join() for t in threads]
+    assert not errors, errors
+    for k, s in enumerate(systems):
+        for o in got[k]:
+            assert torch.equal(o, alone[k]), shapes[k]
+        s.close()
