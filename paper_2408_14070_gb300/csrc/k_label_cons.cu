@@ -69,13 +69,12 @@ __host__ __device__ inline ConsLayout cons_layout(int N, int C) {
     L.sum = o;  o += 8 * (size_t)C;
     L.sum2 = o; o += 8 * (size_t)C;
     L.bp = o;   o += 8 * (size_t)C;
-    L.fD = o;
-    if (N <= RID_BONDED_SMEM_MAX) o += 48 * (size_t)N;
     L.bytes = (o + 15) & ~(size_t)15;
     return L;
 }
 
-// The layout with neighbour lists and all bonded slots (N up to RID_BONDED_SMEM_MAX).  The pre-step
+// The layout with neighbour lists and all bonded slots (N up to RID_BONDED_SMEM_MAX, which fits with every
+// CV count; the one above serves longer chains).  The pre-step
 // positions share the slots' space: those are written and read inside one force evaluation.
 constexpr int CONS_SMEM_MAX = 225 * 1024;
 __host__ __device__ inline ConsLayout cons_layout_lists(int N, int C) {
@@ -175,14 +174,12 @@ __device__ void cons_forces_lists(const SysDev& S, const ConsLayout& L, unsigned
     }
 }
 
-// Force field (bonded + culled LJ) of every bead at xs -> fs.
-__device__ void cons_forces(const SysDev& S, float4* xs, float4* cbox, float3* fD, float4* fs,
-                            unsigned (*keep_s)[LJ_MAX_MASK_WORDS], bool bsm, int nclus, int& bad) {
+// Force field (bonded + culled LJ) of every bead at xs -> fs, for chains too long for lists and slots.
+__device__ void cons_forces(const SysDev& S, float4* xs, float4* cbox, float4* fs,
+                            unsigned (*keep_s)[LJ_MAX_MASK_WORDS], int nclus, int& bad) {
     const int N = S.N, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nwords = (nclus + 31) / 32;
     lj_cluster_boxes(xs, N, cbox);
-    if (bsm)
-        for (int t = tid; t < N; t += CT) bonded_dihedrals_to_smem(S, xs, t, fD);
     __syncthreads();
     const bool sig1 = S.sig2 == 1.0f;
     const float lj_s = -S.lj_eps24;
@@ -204,7 +201,7 @@ __device__ void cons_forces(const SysDev& S, float4* xs, float4* cbox, float3* f
                                         fz, el);
         __syncwarp();
         if (act) {
-            const float3 fb = bsm ? bonded_gather_hybrid(S, xs, i, fD) : bonded_force_on(S, xs, i);
+            const float3 fb = bonded_force_on(S, xs, i);
             const float4 f = make_float4(fmaf(lj_s, fx, fb.x), fmaf(lj_s, fy, fb.y), fmaf(lj_s, fz, fb.z), 0.0f);
             bad |= !(isfinite(f.x) && isfinite(f.y) && isfinite(f.z));
             fs[i] = f;
@@ -267,8 +264,6 @@ __global__ void __launch_bounds__(CT, LISTS ? 4 : 1) k_label_cons(ConsArgs A) {
     double* sum = reinterpret_cast<double*>(smem + L.sum);
     double* sum2 = reinterpret_cast<double*>(smem + L.sum2);
     double* bp = reinterpret_cast<double*>(smem + L.bp);
-    float3* fD = reinterpret_cast<float3*>(smem + L.fD);
-    const bool bsm = N <= RID_BONDED_SMEM_MAX;
     const long long base = (long long)r * N;
     const float* d0 = A.d0 + (long long)r * C;
     const float kick = S.half_dt * S.inv_mass, h = S.half_dt;
@@ -308,7 +303,7 @@ __global__ void __launch_bounds__(CT, LISTS ? 4 : 1) k_label_cons(ConsArgs A) {
     __syncthreads();
     auto forces = [&](bool first) {
         if (LISTS) cons_forces_lists(S, L, smem, keep_s, first, bad);
-        else cons_forces(S, xs, cbox, fD, fs, keep_s, bsm, L.nclus, bad);
+        else cons_forces(S, xs, cbox, fs, keep_s, L.nclus, bad);
     };
     forces(true);
 
@@ -405,15 +400,16 @@ __global__ void __launch_bounds__(CT, LISTS ? 4 : 1) k_label_cons(ConsArgs A) {
 
 }  // namespace
 
-size_t rid_label_cons_smem(int N, int C) { return cons_layout(N, C).bytes; }
+size_t rid_label_cons_smem(int N, int C) {
+    return N <= RID_BONDED_SMEM_MAX ? cons_layout_lists(N, C).bytes : cons_layout(N, C).bytes;
+}
 
 cudaError_t rid_launch_label_cons(const SysDev& S, int R, int C, int B, long long n_steps, long long n_equil,
                                   uint32_t step0, float kT, const float4* x0, const float4* v0, const int2* pairs,
                                   const float* d0, double* bsum, double* mf, double* se, double* sd, float4* x_out,
                                   float4* v_out, int* bad, cudaStream_t st) {
-    const size_t with_lists = S.N <= RID_BONDED_SMEM_MAX ? cons_layout_lists(S.N, C).bytes : 0;
-    const bool lists = with_lists && with_lists <= (size_t)CONS_SMEM_MAX;
-    const size_t smem = lists ? with_lists : rid_label_cons_smem(S.N, C);
+    const bool lists = S.N <= RID_BONDED_SMEM_MAX;
+    const size_t smem = rid_label_cons_smem(S.N, C);
     const auto kern = lists ? k_label_cons<true> : k_label_cons<false>;
     static RidOnce once[2];
     if (const cudaError_t e = rid_opt_in(once[lists], RID_SMEM_MOST, kern)) return e;

@@ -477,7 +477,7 @@ size_t rid_mlp_tc_cluster_smem_bytes(const TcArgs& P) {
 cudaError_t rid_launch_mlp_tc_cluster(const TcArgs& P, const CUtensorMap& big, const CUtensorMap& small,
                                       cudaStream_t s) {
     if (P.ngemm != P.L && P.ngemm != 2 * P.L) return cudaErrorInvalidValue;
-    if (P.csize != 2 && P.csize != 4) return cudaErrorInvalidValue;
+    if (P.csize != 4) return cudaErrorInvalidValue;
     if (P.resnet && !P.rsave) return cudaErrorInvalidValue;
     const size_t smem = rid_mlp_tc_cluster_smem_bytes(P);
     const int v = (P.geb[0] == 1 ? 1 : 0) + (P.resnet ? 2 : 0);

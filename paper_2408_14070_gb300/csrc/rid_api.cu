@@ -93,13 +93,14 @@ struct TcVariant {
     int gN[2 * RID_MAX_LAYERS] = {0}, gKp[2 * RID_MAX_LAYERS] = {0}, geb[2 * RID_MAX_LAYERS] = {0};
     DevBuf blob, wscale;
     CUtensorMap big{}, small{};
-    // cluster variant (k_mlp_tc_cluster, size 4): each GEMM's output columns split over
-    // csize = 2 or 4 CTAs; index 1 = two CTAs (which sizes rid_set_mlp_cluster takes;
-    // k_mlp_tc_pair runs), 2 = four.  The cluster size in use
-    // is chosen by timing the force evaluation at each new walker count.
+    // cluster sizes 2 (index 1) and 4 (index 2) that rid_set_mlp_cluster takes for this
+    // shape: those whose column split, with two operand buffers a CTA, fits in shared
+    // memory.  (Size 4 is that split, k_mlp_tc_cluster.  Size 2 is k_mlp_tc_pair, which
+    // fits every shape; what a caller could pin has stayed the same.)
     bool cl_ok[3] = {false, false, false};
-    int cl_stages[3] = {0, 0, 0}, cl_acc_cols[3] = {0, 0, 0}, cl_tmem_cols[3] = {0, 0, 0};
-    unsigned cl_stage_bytes[3] = {0, 0, 0};
+    int cl_stages = 0, cl_acc_cols = 0, cl_tmem_cols = 0;   // of size 4
+    unsigned cl_stage_bytes = 0;
+    // The cluster size in use is chosen by timing the force evaluation at each new walker count.
     int csize = 1, cs_W = -1;
     int used_cs = 0;   // cluster size of the last launch (0: none yet)
     // small-batch kernel (k_mlp_tc_small): [k][cs], k = 0, 1, 2 for 16, 32, 64
@@ -491,12 +492,12 @@ static int build_tc_variant(rid_system* sys, const std::vector<float>& W, long l
         const size_t fixc = 1024 + 2 * (size_t)V.Kpmax * 256u + sizeof(float) * (size_t)(L + 1) * H;
         const unsigned sb = (unsigned)nsl * 128u;
         V.cl_ok[k] = fixc + 2 * (size_t)sb <= budget && nsl <= 256;
-        if (!V.cl_ok[k]) continue;
-        V.cl_stage_bytes[k] = sb;
-        V.cl_stages[k] = (int)std::min<size_t>((budget - fixc) / sb, TC_MAX_STAGES);
-        V.cl_acc_cols[k] = (nsl + 31) / 32 * 32;
-        V.cl_tmem_cols[k] = 32;
-        while (V.cl_tmem_cols[k] < 2 * V.cl_acc_cols[k]) V.cl_tmem_cols[k] *= 2;
+        if (cs < 4 || !V.cl_ok[k]) continue;
+        V.cl_stage_bytes = sb;
+        V.cl_stages = (int)std::min<size_t>((budget - fixc) / sb, TC_MAX_STAGES);
+        V.cl_acc_cols = (nsl + 31) / 32 * 32;
+        V.cl_tmem_cols = 32;
+        while (V.cl_tmem_cols < 2 * V.cl_acc_cols) V.cl_tmem_cols *= 2;
     }
     // small-batch variants (BF16 only: the transposed GEMMs take the forward
     // weights as the A operand in their BF16 image), per MMA width and number
@@ -1013,10 +1014,10 @@ static int launch_mlp(rid_system* sys, int W, int mode, StateDev sd, cudaStream_
             TRY(timed_launch(sys, "k_mlp_tc", st, [&] { le = rid_launch_mlp_tc_pair(P, 64, V.big, V.small, st); }));
         } else {
             P.csize = cs;
-            P.stages = V.cl_stages[2];
-            P.stage_bytes = V.cl_stage_bytes[2];
-            P.acc_cols = V.cl_acc_cols[2];
-            P.tmem_cols = V.cl_tmem_cols[2];
+            P.stages = V.cl_stages;
+            P.stage_bytes = V.cl_stage_bytes;
+            P.acc_cols = V.cl_acc_cols;
+            P.tmem_cols = V.cl_tmem_cols;
             P.nacc = 2;
             TRY(timed_launch(sys, "k_mlp_tc", st, [&] { le = rid_launch_mlp_tc_cluster(P, V.big, V.small, st); }));
         }
