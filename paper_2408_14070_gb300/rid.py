@@ -192,18 +192,6 @@ def _check(code: int):
 
 
 # ---------------------------------------------------------------------------
-_WRITEABLE, _WARN_ON_WRITE = 0x400, 0x80000000     # bits of ndarray.flags.num
-
-
-def _host_address(a):
-    """Address of a numpy array's first element (the buffer export is several
-    times cheaper than ndarray.ctypes; it needs a writable, non-empty array, and
-    numpy warns when it exports one that broadcast_arrays made)."""
-    if a.size and a.flags.num & (_WRITEABLE | _WARN_ON_WRITE) == _WRITEABLE:
-        return C.addressof(C.c_char.from_buffer(a))
-    return a.ctypes.data
-
-
 class _Args:
     """Collects array pointers of one call and checks they share a memory side."""
 
@@ -219,11 +207,14 @@ class _Args:
         if a is None:
             return None
         if isinstance(a, np.ndarray):
-            if a.dtype != dtype or not a.flags.c_contiguous:
+            flags, n, side = a.flags.num, a.size, RID_MEM_HOST     # 0x1 C-contiguous, 0x400 writable
+            if a.dtype != dtype or not flags & 0x1:
                 raise TypeError(f"expected a C-contiguous numpy array of {np.dtype(dtype)}")
-            if writable and not a.flags.writeable:
+            if writable and not flags & 0x400:
                 raise ValueError("output array is read-only")
-            n, side, p = a.size, RID_MEM_HOST, _host_address(a)
+            # The buffer export is several times cheaper than ndarray.ctypes.  It needs a writable, non-empty
+            # array, and numpy warns when it exports one that broadcast_arrays made (0x80000000).
+            p = C.addressof(C.c_char.from_buffer(a)) if n and flags & 0x80000400 == 0x400 else a.ctypes.data
         elif hasattr(a, "data_ptr"):          # torch tensor
             import torch
             want = {np.float32: torch.float32, np.float64: torch.float64, np.uint32: torch.uint32,
