@@ -768,7 +768,7 @@ def run_paper_network(rid, torch, steps, seed=21):
                  "kernels_ms": kern}
             if name != "fp32":
                 r["roofline"] = tensor_roofline(flops, kern["k_mlp_tc"], fp8_forward=name == "fp8")
-                r["mlp_kernel"] = mlp_kernel_desc(system)
+                r["mlp_kernel"] = mlp_kernel_desc(system, W, H, bf16=name == "bf16")
             res[name] = r
         if name == "bf16":
             # the paper's walker count: step latency
@@ -777,7 +777,7 @@ def run_paper_network(rid, torch, steps, seed=21):
                 x12 = xd[:12].contiguous()
                 ms12, kern12 = _timed_steps(torch, system, x12, stream, steps, flush)
                 res["bf16_12_walkers"] = {"ms_per_step": ms12 / steps, "kernels_ms": kern12,
-                                          "mlp_kernel": mlp_kernel_desc(system, 12)}
+                                          "mlp_kernel": mlp_kernel_desc(system, 12, H)}
             res["bf16_12_walkers_ms_per_step"] = ms12 / steps
     for name in ("bf16", "fp8"):
         d = (grads[name] - grads["fp32"]).norm(dim=1) / grads["fp32"].norm(dim=1).clamp_min(1e-30)
@@ -786,17 +786,31 @@ def run_paper_network(rid, torch, steps, seed=21):
     return res
 
 
-def mlp_kernel_desc(system, walkers=None, bf16=True):
-    """The tensor-core ensemble kernel variant of the system's last launch
-    (BF16 ensembles at up to 16 walkers run the small-batch kernel)."""
-    cs = system.mlp_cluster()
+def mlp_kernel(cs, walkers, width, bf16=True):
+    """The ensemble kernel that a call of `walkers` walkers on an ensemble of this
+    width launches at cluster size cs (rid_get_mlp_cluster; 0: FP32), which is
+    the name of its source file: a one-tile CTA up to 128 walkers and width
+    256, a CTA pair otherwise and at size 2, the column split at size 4; BF16
+    ensembles at up to 16 walkers run the small-batch kernel."""
     if cs == 0:
-        return "FP32 SIMT (k_mlp_fp32)"
-    if walkers is not None and walkers <= 16 and bf16:
-        return f"k_mlp_tc_small: GEMMs transposed, 128-output tiles over clusters of {cs} CTAs per member"
-    if cs == 1:
-        return "k_mlp_tc: one CTA per 128-walker tile and member"
-    return f"k_mlp_tc_cluster: clusters of {cs} CTAs per 128-walker tile and member"
+        return "k_mlp_fp32"
+    if walkers <= 16 and bf16:
+        return "k_mlp_tc_small"
+    if cs == 4:
+        return "k_mlp_tc_cluster"
+    return "k_mlp_tc" if cs == 1 and walkers <= 128 and width <= 256 else "k_mlp_tc_pair"
+
+
+def mlp_kernel_desc(system, walkers, width, bf16=True):
+    """The ensemble kernel variant of the system's last launch, in words."""
+    cs = system.mlp_cluster()
+    name = mlp_kernel(cs, walkers, width, bf16)
+    rows = 128 if cs == 1 and walkers > 128 else 64
+    return {"k_mlp_fp32": "FP32 SIMT (k_mlp_fp32)",
+            "k_mlp_tc_small": f"{name}: GEMMs transposed, 128-output tiles over clusters of {cs} CTAs per member",
+            "k_mlp_tc_cluster": f"{name}: clusters of {cs} CTAs per 128-walker tile and member",
+            "k_mlp_tc": f"{name}: one CTA per 128-walker tile and member",
+            "k_mlp_tc_pair": f"{name}: pairs of CTAs of {rows} walkers each per member"}[name]
 
 
 def run_tiny(rid, torch, seed=1):
@@ -1095,8 +1109,8 @@ def main():
         pass
     tkey = top
     if top == "k_mlp_tc":
-        # the variant the tuner kept names the source and the traffic record
-        tkey = "k_mlp_tc" if system.mlp_cluster() == 1 else "k_mlp_tc_cluster"
+        # the variant that ran names the source and the traffic record
+        tkey = mlp_kernel(system.mlp_cluster(), W, wl["width"])
         work, src = mlp_flops_per_walker_step(wl) * W, tkey + ".cu"
         peak = peaks.get("bf16_tflops")
         roof = {"bound": "tensor", "unit": "TFLOP/s", "peak": peak if peak else 1900.0,
@@ -1161,7 +1175,7 @@ def main():
                       "n_beads": wl["n_beads"], "n_cv": wl["n_cv"], "ensemble": f"{wl['n_models']}x"
                       f"[{2 * wl['n_cv']}-{wl['width']}x{wl['n_layers']}-1]",
                       "mlp_precision": args.precision, "forces_integrator": "f32",
-                      "mlp_kernel": mlp_kernel_desc(system), "ff_cta_threads": system.ff_threads(),
+                      "mlp_kernel": mlp_kernel_desc(system, W, wl["width"]), "ff_cta_threads": system.ff_threads(),
                       "l2": "flushed (256 MiB write) before every timed step; each step timed alone",
                       "parallelism": f"walkers sharded, {world} independent rank(s)"},
            "roofline": roofline, "e2e": e2e, "gpu_launches": launches, "clocks": clk.summary(),

@@ -139,3 +139,15 @@ def test_reference_arm_line_on_rank_zero(B, monkeypatch, capsys):
     assert line["cpu_baseline"]["kind"] == "oracle" and line["cpu_baseline"]["cores"] >= 1
     assert line["e2e"] == {"value": line["value"], "unit": "walker-steps/s", "h2d_bytes_per_step": 0,
                            "d2h_bytes_per_step": 0}
+
+
+def test_the_ensemble_kernel_named_is_the_one_that_runs(B):
+    # sizes as rid_set_mlp_cluster documents them
+    assert B.mlp_kernel(0, 1024, 256) == "k_mlp_fp32"
+    assert B.mlp_kernel(1, 1024, 256) == B.mlp_kernel(2, 1024, 256) == B.mlp_kernel(2, 100, 64) == "k_mlp_tc_pair"
+    assert B.mlp_kernel(1, 128, 256) == "k_mlp_tc" and B.mlp_kernel(1, 128, 300) == "k_mlp_tc_pair"
+    assert B.mlp_kernel(4, 1024, 256) == "k_mlp_tc_cluster"
+    assert B.mlp_kernel(3, 12, 300) == "k_mlp_tc_small" and B.mlp_kernel(1, 12, 300, bf16=False) == "k_mlp_tc_pair"
+    csrc = os.path.join(ROOT, "paper_2408_14070_gb300", "csrc")
+    for name in ("k_mlp_fp32", "k_mlp_tc_pair", "k_mlp_tc", "k_mlp_tc_cluster", "k_mlp_tc_small"):
+        assert os.path.exists(os.path.join(csrc, name + ".cu"))
