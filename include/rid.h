@@ -475,13 +475,17 @@ RID_API int64_t rid_launch_count(rid_system* sys);
 
 /*
  * Cluster size of the tensor-core ensemble kernel (BF16 / FP8 ensembles; no
- * counterpart in the paper, a tuning control).  The kernel splits every
- * GEMM's output columns over csize CTAs of a thread-block cluster (1: one CTA
- * per 128-walker tile and member; 2 or 4: the columns split over a cluster,
- * the next layer's operand exchanged through distributed shared memory).
- * csize = 0 (the default) lets the library time the force evaluation with
- * each eligible size at the first evaluation of every new walker count and
- * keep the fastest.  Every size gives the same results bit for bit.  BF16
+ * counterpart in the paper, a tuning control): how many CTAs share a tile of
+ * 128 walkers of one member.  1: one CTA (with two tiles or more, CTA pairs of
+ * two tiles whose MMAs share the weights; a single tile of an ensemble wider
+ * than 256 takes a pair of 64 walkers each).  2: a pair of 64 walkers each.  4:
+ * every GEMM's output columns split over four CTAs, the next layer's operand
+ * exchanged through distributed shared memory.
+ * csize = 0 (the default): at the first evaluation of a new walker count whose
+ * pairs of 64 walkers fit the GPU at once, the library times the force
+ * evaluation with sizes 1 and 2 and keeps 2 if it is 8% faster, else 1; larger
+ * counts take 1; member values alone (MCMC) take 2 while the pairs fit, else 1.
+ * Every size gives the same results bit for bit.  BF16
  * ensembles evaluated for at most 16 walkers run a small-batch kernel instead
  * (the GEMMs transposed, each GEMM's 128-output tiles split over a cluster of
  * one CTA per tile, at most 4, or at most csize CTAs when csize is fixed; no
@@ -492,9 +496,9 @@ RID_API int64_t rid_launch_count(rid_system* sys);
  * for the row kernels and nothing is timed: the request loop does not wait on
  * timing runs, and a size timed on an idle GPU is not the one for a shared
  * GPU.
- * Errors: RID_ERR_ARG (csize not 0, 1, 2 or 4); a size the ensemble's shape
- * does not allow (shared memory) fails with RID_ERR_ARG at the next
- * evaluation.
+ * Errors: RID_ERR_ARG (csize not 0, 1, 2 or 4); a fixed size of 2 or 4 fails
+ * with RID_ERR_ARG at the next evaluation where two operand buffers of 128
+ * walkers and the weights of a column split do not fit in shared memory.
  */
 RID_API int rid_set_mlp_cluster(rid_system* sys, int32_t csize);
 

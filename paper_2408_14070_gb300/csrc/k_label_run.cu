@@ -1,6 +1,7 @@
 // k_label_run.cu -- restrained label runs, one CTA per run with all of its
-// steps in one launch: rid_label and rid_label_batch for chains whose bonded
-// slots fit in shared memory (RID_BONDED_SMEM_MAX beads).
+// steps in one launch: rid_label_batch for chains whose bonded slots fit in
+// shared memory (RID_BONDED_SMEM_MAX beads), rid_label for chains below 768
+// beads.
 //
 // The same step as k_label_fused, term for term and in the same order (so the
 // same bits as there and as through the per-step kernels), arranged for the

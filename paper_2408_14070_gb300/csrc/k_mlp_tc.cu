@@ -8,8 +8,9 @@
 // kind is issued.  FP8 weights are stored as W / s_W and the accumulator is
 // scaled back by s_W in the epilogue.
 //
-// Work unit: one CTA = one tile of 128 walkers x one ensemble member.  The
-// chain of 2L GEMMs
+// Work unit: one CTA = one tile of 128 walkers x one ensemble member.  It runs a
+// single tile up to width 256, where two accumulators fit in TMEM; more tiles and
+// wider members take CTA pairs (k_mlp_tc_pair).  The chain of 2L GEMMs
 //   forward  l = 0..L-1 :  Z_l = H_{l-1} W_l^T      (128 x H,   K = D' or H)
 //   backward l = L-1..0 :  G_{l-1} = Delta_l W_l     (128 x fin, K = H)
 // runs with the activation tile (A operand, BF16) resident in shared memory
@@ -67,13 +68,14 @@ __global__ void __maxnreg__(96)
         reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(dsm_raw) + 1023) & ~uintptr_t(1023));
     __shared__ Smem S;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int tile = blockIdx.x, m = blockIdx.y;
+    constexpr int tile = 0;            // a call of more than 128 walkers takes CTA pairs
+    const int m = blockIdx.y;
     const int L = P.L, G = P.ngemm;   // 2L, or L for the member values alone
     unsigned char* Abuf = dsm;                                     // [Kpmax/64][128 rows][128 B]
     unsigned char* stages = dsm + (size_t)P.Kpmax * 256u;          // 128 rows x 2 B per column
     const uint32_t stage_bytes = P.stage_bytes;
     const int NS = P.stages;
-    const int NACC = P.nacc;
+    constexpr int NACC = 2;            // accumulators in TMEM
     volatile int* abort_flag = &S.abort_flag;
 
     if (threadIdx.x == 0) {
@@ -447,6 +449,7 @@ size_t rid_mlp_tc_smem_bytes(const TcArgs& P) {
 
 cudaError_t rid_launch_mlp_tc(const TcArgs& P, const CUtensorMap& big, const CUtensorMap& small, cudaStream_t s) {
     if (P.ngemm != P.L && P.ngemm != 2 * P.L) return cudaErrorInvalidValue;
+    if (P.ntiles != 1 || P.nacc != 2) return cudaErrorInvalidValue;
     if (P.resnet && !P.rsave) return cudaErrorInvalidValue;
     const size_t smem = rid_mlp_tc_smem_bytes(P);
     const int v = (P.geb[0] == 1 ? 1 : 0) + (P.resnet ? 2 : 0);
@@ -454,6 +457,6 @@ cudaError_t rid_launch_mlp_tc(const TcArgs& P, const CUtensorMap& big, const CUt
               : v == 2 ? k_mlp_tc<false, true> : k_mlp_tc<true, true>;
     static RidOnce once[4];
     if (const cudaError_t e = rid_opt_in(once[v], RID_SMEM_MOST, kern)) return e;
-    kern<<<dim3(P.ntiles, P.M, 1), NTHREADS, smem, s>>>(P, big, small);
+    kern<<<dim3(1, P.M, 1), NTHREADS, smem, s>>>(P, big, small);
     return cudaGetLastError();
 }

@@ -1,5 +1,6 @@
 // k_mlp_tc_cluster.cu -- the tcgen05 ensemble MLP with each GEMM's output
-// columns split over a thread-block cluster of S = 2 or 4 CTAs.
+// columns split over a thread-block cluster of S = 4 CTAs: cluster size 4, which
+// runs when a caller pins it (slower than CTA pairs at every size measured).
 //
 // Same arithmetic as k_mlp_tc (BF16 / FP8 operands, FP32 accumulation in
 // TMEM, tanh saved in BF16, optional residual stream in FP32); what differs

@@ -8,7 +8,8 @@
 // for 2 x ROWS walkers: each CTA keeps ROWS rows of the activations in its
 // shared memory and streams half of every weight chunk's rows, and one
 // tcgen05.mma of the even CTA multiplies both CTAs' rows by both halves.
-// Every wait is bounded in time.
+// Every wait on an mbarrier is bounded in time (the TMEM allocation, which waits for
+// CTAs that hold columns to end, and the cluster barriers are not).
 //
 // A GEMM is a serial chain: MMAs, accumulator to the epilogue, element work,
 // operand back to the MMAs.  At 512 columns the 128 KB operand left room for
@@ -84,7 +85,8 @@ __device__ __forceinline__ void pair_tma_load(uint32_t dst, const CUtensorMap* m
 // Hand this CTA's rows of an operand to the even CTA, whose MMAs read them: release at cluster scope of
 // shared memory alone, before a relaxed arrive (the writers have handed it to the async proxy already).  An
 // arrive that releases all memory costs half a microsecond a GEMM here, also from a thread that has written
-// nothing: 30.5 -> 34.2 us a launch (128 walkers of 4 x 40-256x4-1), 30.6 with this fence.
+// nothing: 30.5 -> 34.2 us a launch (128 walkers of 4 x 40-256x4-1), 30.6 with this fence.  (The default scope
+// took 0.9 us less of a step's 49.9, 1024 walkers of 200 beads, and orders the arriving CTA only.)
 __device__ __forceinline__ void pair_arrive(uint32_t local_bar) {
     asm volatile("fence.release.sync_restrict::shared::cta.cluster;" ::: "memory");
     asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(mapa(local_bar, 0)) : "memory");

@@ -42,8 +42,8 @@ struct FusedArgs {
 };
 
 // One CTA per run, the terms of a step as tasks of its warps (k_label_run).
-// Shared memory for N beads and C CVs, 0 when it does not fit (from about 870
-// beads on):
+// Shared memory for N beads and C CVs, 0 when it does not fit: beyond 1024 beads
+// (RID_BONDED_SMEM_MAX), and at 1021 to 1024 beads with 128 CVs.
 size_t rid_label_run_smem(int N, int C);
 // CTA size for `runs` runs of chains of up to N beads and smem bytes of shared
 // memory: a warp for every task of a step, up to 16, while that takes as few

@@ -42,7 +42,7 @@ struct TcArgs {
     const float* wscale;     // [M][2L] weight scale of every GEMM (1 for BF16)
     int resnet;              // h_l = h_{l-1} + tanh(z_l) for l >= 1
     float* rsave;            // resnet: [M][ntiles][H/8][128][8] FP32, h_l forward, dA/dh_l backward
-    int csize;               // cluster variant: CTAs splitting each GEMM's output columns (2 or 4)
+    int csize;               // cluster variant: CTAs splitting each GEMM's output columns (4)
     int ngemm;               // GEMMs to run: 2L (forward and input gradient) or L (forward only:
                              // member values, gradA untouched)
 };
