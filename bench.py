@@ -1131,7 +1131,7 @@ def main():
         work, src = pair_flops_per_walker_step(wl) * W, "k_step.cu"
         roof = {"bound": "alu", "unit": "TFLOP/s", "peak": fp32_peak(torch)[0], "peak_source": fp32_peak(torch)[1]}
         achieved = work / (avg_ms / 1e3) / 1e12
-    roofline = {"kernel": top, "bound": roof["bound"], "achieved": achieved, "peak": roof["peak"],
+    roofline = {"kernel": tkey, "bound": roof["bound"], "achieved": achieved, "peak": roof["peak"],
                 "unit": roof["unit"], "frac": achieved / roof["peak"] if roof["peak"] else None,
                 "traffic": traffic_for(tkey, src, WORKLOAD), "work_per_launch": work, "source": src,
                 "avg_launch_ms": avg_ms, "peak_source": roof["peak_source"],
