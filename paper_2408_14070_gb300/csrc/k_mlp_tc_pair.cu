@@ -86,8 +86,13 @@ __device__ __forceinline__ void pair_tma_load(uint32_t dst, const CUtensorMap* m
 // shared memory alone, before a relaxed arrive (the writers have handed it to the async proxy already).  An
 // arrive that releases all memory costs half a microsecond a GEMM here, also from a thread that has written
 // nothing: 30.5 -> 34.2 us a launch (128 walkers of 4 x 40-256x4-1), 30.6 with this fence.  (The default scope
-// took 0.9 us less of a step's 49.9, 1024 walkers of 200 beads, and orders the arriving CTA only.)
-__device__ __forceinline__ void pair_arrive(uint32_t local_bar) {
+// took 0.4 us less of a step's 49.8, 1024 walkers of 200 beads, and orders the arriving CTA only, which is why
+// the even CTA's own rows take it: with the fence in both CTAs a step took 50.1 us.)
+__device__ __forceinline__ void pair_arrive(uint32_t local_bar, uint32_t rank) {
+    if (rank == 0) {                  // its own rows: the reader is in this CTA
+        mbar_arrive(local_bar);
+        return;
+    }
     asm volatile("fence.release.sync_restrict::shared::cta.cluster;" ::: "memory");
     asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(mapa(local_bar, 0)) : "memory");
 }
@@ -463,7 +468,7 @@ __global__ void __maxnreg__(96)
         const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16);
         const int H = P.H;
         const uint32_t a_bar = smem_u32(&S.a_full);
-        if (lane == 0) pair_arrive(a_bar);       // the input is in place
+        if (lane == 0) pair_arrive(a_bar, rank);       // the input is in place
         __nv_bfloat16* tsave_tile = P.tsave + ((size_t)m * P.ntiles + tile) * (size_t)L * 128 * H;
         // residual stream of a resnet ensemble: h_l (forward) and dA/dh_l (backward)
         // in FP32, one [H/8][128][8] block per tile and member, overwritten in place
@@ -650,7 +655,7 @@ __global__ void __maxnreg__(96)
                 fence_async_smem();
                 fence_before();
                 __syncwarp();
-                if (lane == 0) pair_arrive(a_bar);
+                if (lane == 0) pair_arrive(a_bar, rank);
                 if (late) {
                     // only this thread writes these operand columns again, after the GEMM that reads them
                     for (int i = i0; i < i1; ++i) {
