@@ -259,8 +259,9 @@ __global__ void __launch_bounds__(NT, RPT >= 4 && CPT == 8 ? 1 : 2) k_mlp_fp32(M
     const Lane t = lane_of<WCN>();
     const int own = t.rg * GS;                          // this thread's slots of a row
     // saved tanh: rows of the tile's slots; a last tile of 64 that holds 32 walkers or fewer keeps half of them
-    const int tw = RPT == 8 && R == 64 && W - w0 <= 32 ? 32 : S::SLOTS;
-    const bool keep = own < tw;
+    constexpr bool halves = RPT == 8 && R == 64;
+    const int tw = halves && W - w0 <= 32 ? 32 : S::SLOTS;
+    const bool keep = !halves || own < tw;
     const size_t wst = RPT == 7 ? (size_t)gridDim.x * S::SLOTS : f32_walkers(W);
     float* hs = BWD ? E.hs + (m * wst + (size_t)blockIdx.x * S::SLOTS) * (size_t)L * H + own : nullptr;
 
